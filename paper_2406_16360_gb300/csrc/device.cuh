@@ -28,12 +28,6 @@
 #else
 #define MR_TRACE_BOUNDS __launch_bounds__(256)
 #endif
-#ifndef MR_REFILL
-#define MR_REFILL 1  // batched wavefront: shadow rays traced by lane-refilling warps
-#endif
-#ifndef MR_REFILL_CLOSEST
-#define MR_REFILL_CLOSEST 1  // ... and continuation rays (at 64 registers: 6-8% faster than k_wclosest)
-#endif
 #ifndef MR_DFS_NODES
 #define MR_DFS_NODES 1  // traversal nodes in depth-first preorder (else the builders' order)
 #endif
@@ -48,10 +42,22 @@
 #define MR_CLOSEST_REFILL_MINB 4  // its register cap: four 256-thread blocks per SM (64 registers)
 #endif
 #ifndef MR_REFILL_STEPS
-#define MR_REFILL_STEPS 16  // node visits between refill checks
+#define MR_REFILL_STEPS 12  // node visits between refill checks
 #endif
 #ifndef MR_REFILL_MIN
-#define MR_REFILL_MIN 8  // idle lanes that trigger a refill
+#define MR_REFILL_MIN 6  // idle lanes that trigger a refill
+#endif
+// Lane-refilling traversal (trav_warp), measured on 12 views of config 3 (12 launches of
+// continuation rays / 16 of shadow rays, ms) against leaves tested on the spot, 38.6 / 41.6:
+// tests once 16 lanes wait 36.7 / 43.6, once 8 do 33.7 / 39.8; with room for six leaves, a
+// 16-entry shared stack (more L1 left for nodes) and refills every 12 visits at 6 idle lanes
+// 32.9 / 39.0. Few waiting lanes are enough because the stage is bound by the latency and the L1
+// wavefronts of its loads, not by issue slots alone.
+#ifndef MR_PEND
+#define MR_PEND 6  // leaves a lane may put aside
+#endif
+#ifndef MR_PEND_MIN
+#define MR_PEND_MIN 8  // lanes with such a leaf that start the triangle tests, whatever the others do
 #endif
 #ifndef MR_CAND_UNROLL
 #define MR_CAND_UNROLL 1
@@ -64,7 +70,7 @@
 // deeper entries in a small local array; an LBVH over 64-bit unique keys is at most 63 deep
 // (a clustering tree deeper than the stack is not used)
 #ifndef MR_SSTACK
-#define MR_SSTACK 32
+#define MR_SSTACK 16
 #endif
 #define MR_LSTACK (64 - MR_SSTACK)
 static_assert(MR_SSTACK >= 8 && MR_SSTACK <= 56, "MR_SSTACK out of range");
@@ -889,19 +895,30 @@ __device__ __forceinline__ int trace_as(const SceneDev& s, float3 o, float3 d, i
     return traverse<ANY>(s, o, d, skip, tmin, tmax, best, sstk, blockDim.x, ntri);
 }
 
-// The same traversal as a resumable state, for kernels that interleave the rays of a warp's
-// lanes and hand a finished lane a new ray: trav_begin sets a ray up, trav_run advances it by
-// at most `steps` node visits and returns true when it is done (result in T.best; T.visited =
-// -1 when the iteration cap was reached). The stack is the thread's shared column plus `lstk`.
+// The same traversal as a resumable warp-wide state, for kernels that interleave the rays of a
+// warp's lanes and hand a finished lane a new ray: trav_begin sets a lane's ray up, trav_warp
+// (called by all 32 lanes) advances every lane's ray by at most `steps` node visits. A leaf that a
+// lane reaches is not tested on the spot but put aside (up to MR_PEND of them, in the thread's
+// shared column behind its stack) while the warp goes on visiting nodes; the triangle tests run
+// once MR_PEND_MIN lanes have one, or half as many lanes as can still go on (the last rays of a
+// queue, few to a warp, are thus tested almost on the spot).
 struct Trav {
     float3 o, d, inv, oi;
     float tmin;
-    int skip, node, sp, visited;  // node < 0: done
+    int skip, node, sp, pend, left;  // node < 0 and pend == 0: done; left: node visits to the cap
+    const float4* nodes;
     Hit best;
+    __device__ __forceinline__ bool done() const { return node < 0 && pend == 0; }
 };
 
+// Putting leaves aside changes no hit (a triangle is tested whenever its leaf's box passes, and
+// the closest of them, or any, is kept), but best.t shrinks a little later, so a ray may visit a
+// few more nodes. Under a caller's own iteration cap leaves are therefore tested before the next
+// visit (ahead = false), so that a ray reaches the cap exactly when traverse() would.
+__device__ __forceinline__ bool trav_ahead(const SceneDev& s) { return s.trav_cap <= 0; }
+
 __device__ __forceinline__ void trav_begin(const SceneDev& s, Trav& T, float3 o, float3 d, int skip, float tmin,
-                                           float tmax, int* ntri)
+                                           float tmax)
 {
     T.best.t = tmax;
     T.best.tri = -1;
@@ -913,84 +930,80 @@ __device__ __forceinline__ void trav_begin(const SceneDev& s, Trav& T, float3 o,
     T.tmin = tmin;
     T.skip = skip;
     T.sp = 0;
-    T.visited = 0;
+    T.pend = 0;
+    T.left = trav_cap_of(s);
+    T.nodes = s.nodes;
     T.node = 0;
     if (s.n_tris <= 0) {
         T.node = -1;
     } else if (s.n_tris == 1) {
-        if (ntri) ++*ntri;
         test_leaf(s, 0, o, d, skip, tmin, T.best);
         T.node = -1;
     }
 }
 
 template <bool ANY>
-__device__ __forceinline__ bool trav_run(const SceneDev& s, Trav& T, uint32_t* sstk, int sstride, uint32_t* lstk,
-                                         int steps, int* ntri)
+__device__ __forceinline__ void trav_warp(const SceneDev& s, Trav& T, uint32_t* sstk, int sstride, uint32_t* lstk,
+                                          int steps, bool ahead)
 {
-    if (T.node < 0) return true;
-    const int cap = trav_cap_of(s);
+    const int most = ahead ? MR_PEND - 2 : 0;
     for (int k = 0; k < steps; ++k) {
-        if (++T.visited > cap) {
-            T.best.tri = -1;
-            T.visited = -1;
-            T.node = -1;
-            trav_fail(s);
-            return true;
-        }
-        const int node = T.node;
-        float4 n0, n1, n2;
-        int2 ch;
-        load_node(s.nodes + 4 * (size_t)node, n0, n1, n2, ch);
-        const float tl = slab(f3(n0.x, n0.y, n0.z), f3(n0.w, n1.x, n1.y), T.oi, T.inv, T.tmin, T.best.t);
-        const float tr = slab(f3(n1.z, n1.w, n2.x), f3(n2.y, n2.z, n2.w), T.oi, T.inv, T.tmin, T.best.t);
-        bool gl = tl <= T.best.t, gr = tr <= T.best.t;
-        if (gl && ch.x < 0) {
-            if (ntri) ++*ntri;
-            if (test_leaf(s, ~ch.x, T.o, T.d, T.skip, T.tmin, T.best) && ANY) {
-                T.node = -1;
-                return true;
-            }
-            gl = false;
-        }
-        if (gr && ch.y < 0) {
-            if (ntri) ++*ntri;
-            if (test_leaf(s, ~ch.y, T.o, T.d, T.skip, T.tmin, T.best) && ANY) {
-                T.node = -1;
-                return true;
-            }
-            gr = false;
-        }
-        if (gl && gr) {
-            const bool lfirst = tl <= tr;
-            const int nearc = lfirst ? ch.x : ch.y, farc = lfirst ? ch.y : ch.x;
-            if (T.sp < MR_SSTACK) {
-                sstk[T.sp * sstride] = (uint32_t)farc;
-            } else if (T.sp < MR_SSTACK + MR_LSTACK) {
-                lstk[T.sp - MR_SSTACK] = (uint32_t)farc;
-            } else {
+        if (T.node >= 0 && T.pend <= most) {
+            if (--T.left < 0) {
                 T.best.tri = -1;
-                T.visited = -1;
                 T.node = -1;
+                T.pend = 0;
                 trav_fail(s);
-                return true;
+            } else {
+                float4 n0, n1, n2;
+                int2 ch;
+                load_node(T.nodes + 4 * (size_t)T.node, n0, n1, n2, ch);
+                const float tl = slab(f3(n0.x, n0.y, n0.z), f3(n0.w, n1.x, n1.y), T.oi, T.inv, T.tmin, T.best.t);
+                const float tr = slab(f3(n1.z, n1.w, n2.x), f3(n2.y, n2.z, n2.w), T.oi, T.inv, T.tmin, T.best.t);
+                bool gl = tl <= T.best.t, gr = tr <= T.best.t;
+                if (gl && ch.x < 0) {
+                    sstk[(MR_SSTACK + T.pend) * sstride] = (uint32_t)~ch.x;
+                    ++T.pend;
+                    gl = false;
+                }
+                if (gr && ch.y < 0) {
+                    sstk[(MR_SSTACK + T.pend) * sstride] = (uint32_t)~ch.y;
+                    ++T.pend;
+                    gr = false;
+                }
+                if (gl && gr) {
+                    const bool lfirst = tl <= tr;
+                    const int nearc = lfirst ? ch.x : ch.y, farc = lfirst ? ch.y : ch.x;
+                    T.node = nearc;
+                    if (T.sp < MR_SSTACK) sstk[T.sp * sstride] = (uint32_t)farc;
+                    else if (T.sp < MR_SSTACK + MR_LSTACK) lstk[T.sp - MR_SSTACK] = (uint32_t)farc;
+                    else T.left = 0;  // deeper than any tree the builders keep: a malformed tree, ended as by the cap
+                    ++T.sp;
+                } else if (gl || gr) {
+                    T.node = gl ? ch.x : ch.y;
+                } else if (T.sp == 0) {
+                    T.node = -1;
+                } else {
+                    --T.sp;
+                    T.node = (int)(T.sp < MR_SSTACK ? sstk[T.sp * sstride] : lstk[T.sp - MR_SSTACK]);
+                }
             }
-            ++T.sp;
-            T.node = nearc;
-        } else if (gl) {
-            T.node = ch.x;
-        } else if (gr) {
-            T.node = ch.y;
-        } else {
-            if (T.sp == 0) {
-                T.node = -1;
-                return true;
+        }
+        const unsigned wait = __ballot_sync(MR_FULL, T.pend > 0);
+        const unsigned can = __ballot_sync(MR_FULL, T.node >= 0 && T.pend <= most);
+        if ((wait | can) == 0u) break;  // every lane is done
+        const int n_wait = __popc(wait);
+        if (n_wait >= MR_PEND_MIN || 2 * n_wait >= __popc(can) || !ahead) {
+            if (T.pend > 0) {
+                --T.pend;
+                const int leaf = (int)sstk[(MR_SSTACK + T.pend) * sstride];
+                if (test_leaf(s, leaf, T.o, T.d, T.skip, T.tmin, T.best) && ANY) {
+                    T.node = -1;
+                    T.pend = 0;
+                }
             }
-            --T.sp;
-            T.node = (int)(T.sp < MR_SSTACK ? sstk[T.sp * sstride] : lstk[T.sp - MR_SSTACK]);
         }
     }
-    return false;
 }
 
 // ---------------------------------------------------------------------------------------

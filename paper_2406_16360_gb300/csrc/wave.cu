@@ -567,25 +567,23 @@ __device__ __forceinline__ long long refill(RefillPool& rp, bool has, unsigned i
     return mine;
 }
 
-template <bool COUNT>
 __global__ void __launch_bounds__(256, MR_CLOSEST_REFILL_MINB) k_wclosest_refill(const SceneDev* __restrict__ scenes,
                                                          const ViewDev* __restrict__ views, QueueDev q,
                                                          const unsigned int* count, QueueDev hq,
-                                                         unsigned int* count_hit, unsigned int* fetch,
-                                                         unsigned long long* counters)
+                                                         unsigned int* count_hit, unsigned int* fetch)
 {
     extern __shared__ __align__(16) uint32_t sstk[];
     const unsigned int n = *count;
     uint32_t lstk[MR_LSTACK];
     Trav T;
     T.node = -1;
+    T.pend = T.left = 0;
     bool has = false;
     unsigned int i = 0;
     RefillPool rp{0u, 0u, false};
     float4 qd = make_float4(0.f, 0.f, 0.f, 0.f), qb = qd;
     const SceneDev* sp = scenes;
-    unsigned int n_box = 0;
-    int n_tri = 0;
+    const bool ahead = trav_ahead(*scenes);
     while (true) {
         const long long ni = refill(rp, has, n, fetch);
         if (ni >= 0) {
@@ -594,18 +592,12 @@ __global__ void __launch_bounds__(256, MR_CLOSEST_REFILL_MINB) k_wclosest_refill
             qd = q.d[i];
             qb = q.b[i];
             sp = scenes + views[__float_as_int(qb.w)].scene;
-            trav_begin(*sp, T, xyz(a), xyz(qd), __float_as_int(a.w), *sp->tmin_dev, __int_as_float(0x7f800000),
-                       COUNT ? &n_tri : nullptr);
+            trav_begin(*sp, T, xyz(a), xyz(qd), __float_as_int(a.w), *sp->tmin_dev, __int_as_float(0x7f800000));
             has = true;
         }
         if (!__any_sync(MR_FULL, has)) break;
-        bool done = false;
-        if (has) {
-            const int v0 = T.visited;
-            done = trav_run<false>(*sp, T, sstk + threadIdx.x, blockDim.x, lstk, MR_REFILL_STEPS,
-                                   COUNT ? &n_tri : nullptr);
-            if (COUNT) n_box += 2u * (unsigned int)max(T.visited - v0, 0);
-        }
+        trav_warp<false>(*sp, T, sstk + threadIdx.x, blockDim.x, lstk, MR_REFILL_STEPS, ahead);
+        const bool done = has && T.done();
         if (__any_sync(MR_FULL, done)) {
             const bool hit = done && T.best.tri >= 0;
             const unsigned int slot = warp_append(hit, count_hit);
@@ -618,14 +610,12 @@ __global__ void __launch_bounds__(256, MR_CLOSEST_REFILL_MINB) k_wclosest_refill
             if (done) has = false;
         }
     }
-    if (COUNT) flush_work(counters, CNT_CBOX, n_box, (unsigned int)n_tri);
 }
 
-template <bool COUNT>
 __global__ void MR_TRACE_BOUNDS k_wshadow_refill(const SceneDev* __restrict__ scenes,
                                                         const ViewDev* __restrict__ views, int b, ShadowDev sq,
                                                         const unsigned int* count, unsigned int* fetch, void* tape,
-                                                        uint64_t ntot, int nvx, unsigned long long* counters)
+                                                        uint64_t ntot, int nvx)
 {
     extern __shared__ __align__(16) uint32_t sstk[];
     const TapeDev tp = tape_of(tape, ntot, nvx);
@@ -633,13 +623,13 @@ __global__ void MR_TRACE_BOUNDS k_wshadow_refill(const SceneDev* __restrict__ sc
     uint32_t lstk[MR_LSTACK];
     Trav T;
     T.node = -1;
+    T.pend = T.left = 0;
     bool has = false;
     unsigned int i = 0;
     RefillPool rp{0u, 0u, false};
     float4 dd = make_float4(0.f, 0.f, 0.f, 0.f), ad = dd;
     const SceneDev* sp = scenes;
-    unsigned int n_box = 0;
-    int n_tri = 0;
+    const bool ahead = trav_ahead(*scenes);
     while (true) {
         const long long ni = refill(rp, has, n, fetch);
         if (ni >= 0) {
@@ -648,17 +638,13 @@ __global__ void MR_TRACE_BOUNDS k_wshadow_refill(const SceneDev* __restrict__ sc
             dd = sq.d[i];
             ad = sq.add[i];
             sp = scenes + views[__float_as_int(ad.w)].scene;
-            trav_begin(*sp, T, xyz(a), xyz(dd), __float_as_int(a.w), *sp->tmin_dev, __int_as_float(0x7f800000),
-                       COUNT ? &n_tri : nullptr);
+            trav_begin(*sp, T, xyz(a), xyz(dd), __float_as_int(a.w), *sp->tmin_dev, __int_as_float(0x7f800000));
             has = true;
         }
         if (!__any_sync(MR_FULL, has)) break;
+        trav_warp<true>(*sp, T, sstk + threadIdx.x, blockDim.x, lstk, MR_REFILL_STEPS, ahead);
         if (has) {
-            const int v0 = T.visited;
-            const bool done = trav_run<true>(*sp, T, sstk + threadIdx.x, blockDim.x, lstk, MR_REFILL_STEPS,
-                                             COUNT ? &n_tri : nullptr);
-            if (COUNT) n_box += 2u * (unsigned int)max(T.visited - v0, 0);
-            if (done) {
+            if (T.done()) {
                 has = false;
                 const uint64_t g = views[__float_as_int(ad.w)].offset + __float_as_uint(dd.w);
                 if (T.best.tri < 0) {
@@ -679,7 +665,6 @@ __global__ void MR_TRACE_BOUNDS k_wshadow_refill(const SceneDev* __restrict__ sc
             }
         }
     }
-    if (COUNT) flush_work(counters, CNT_SBOX, n_box, (unsigned int)n_tri);
 }
 
 // ---- primary visibility by rasterisation ------------------------------------------------
@@ -851,14 +836,12 @@ void mr_wave_record(const SceneDev* scenes, const ViewDev* views, int n_views, u
         interp = interp || hscenes[hviews[i].scene].vnrm != nullptr;
         wide = wide && (hscenes[hviews[i].scene].wnodes != nullptr || hscenes[hviews[i].scene].n_tris < 2);
     }
-    const size_t smem = sizeof(uint32_t) * MR_SSTACK * 256;  // the refilling kernels run 256 threads
+    const size_t smem = sizeof(uint32_t) * (MR_SSTACK + MR_PEND) * 256;  // the refilling kernels run 256 threads
     const size_t stack_c = sizeof(uint32_t) * MR_SSTACK * (size_t)blk_c, stack_s = sizeof(uint32_t) * MR_SSTACK * (size_t)blk_s;
     // the refilling kernels run one resident wave of blocks
     int occ_c = 0, occ_s = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_c, count ? k_wclosest_refill<true> : k_wclosest_refill<false>,
-                                                  256, smem);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_s, count ? k_wshadow_refill<true> : k_wshadow_refill<false>,
-                                                  256, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_c, k_wclosest_refill, 256, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_s, k_wshadow_refill, 256, smem);
     const unsigned grid_c = (unsigned)(sms * (occ_c > 0 ? occ_c : 1));
     const unsigned grid_s = (unsigned)(sms * (occ_s > 0 ? occ_s : 1));
     int pair = 0, cur_b = -1;  // cur_b: the bounce being recorded (-1: ray generation)
@@ -919,9 +902,9 @@ void mr_wave_record(const SceneDev* scenes, const ViewDev* views, int n_views, u
                         scenes, views, vi, first, n, cur.d, keys, counters);
                 }
             }
-            if (MR_REFILL_CLOSEST && b > 0 && !wide)  // primary rays stay coherent in the plain stage kernel
-                (count ? k_wclosest_refill<true> : k_wclosest_refill<false>)<<<grid_c, 256, smem, st>>>(
-                    scenes, views, cur, cnt_in, hq, qc + 3 * b, fetch + 2 * b, counters);
+            // primary rays stay coherent in the plain stage kernel; work is counted there too, ray by ray
+            if (b > 0 && !wide && !count)
+                k_wclosest_refill<<<grid_c, 256, smem, st>>>(scenes, views, cur, cnt_in, hq, qc + 3 * b, fetch + 2 * b);
             else
                 (keys ? (count ? k_wclosest<true, true, false>
                                : (wide ? k_wclosest<false, true, true> : k_wclosest<false, true, false>))
@@ -946,9 +929,9 @@ void mr_wave_record(const SceneDev* scenes, const ViewDev* views, int n_views, u
                 k_whist_miss<<<grid_cap(n, blk_h, cap_h), blk_h, 0, st>>>(first, n, tape, total, hist);
             mark(1, false);
             mark(2, true);
-            if (MR_REFILL && !wide)
-                (count ? k_wshadow_refill<true> : k_wshadow_refill<false>)<<<grid_s, 256, smem, st>>>(
-                    scenes, views, b, sq, qc + 3 * b + 2, fetch + 2 * b + 1, tape, total, nvx, counters);
+            if (!wide && !count)
+                k_wshadow_refill<<<grid_s, 256, smem, st>>>(scenes, views, b, sq, qc + 3 * b + 2, fetch + 2 * b + 1, tape,
+                                                            total, nvx);
             else
                 (count ? k_wshadow<true, false> : (wide ? k_wshadow<false, true> : k_wshadow<false, false>))<<<
                     grid_cap(n, blk_s, cap_s), blk_s, stack_s, st>>>(
