@@ -331,7 +331,7 @@ extern "C" mirres_status mirres_bvh_build(mirres_scene* s, void* stream)
     const cudaStream_t st = as_stream(stream);
     MR_TRY(mr_bvh_build(s, st));
     MR_TRY(mr_env_build(s, st));
-    s->ctx->host_launches += 24;
+    s->ctx->host_launches += 20;
     s->built = true;
     return MIRRES_OK;
 }

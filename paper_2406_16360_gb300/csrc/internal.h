@@ -104,17 +104,15 @@ struct mirres_scene {
     int32_t* ploc_state = nullptr;   // [4]: cluster count and next free node id, by iteration parity
     // env tables
     double* env_w = nullptr;         // [eh][ew]
+    double* env_before = nullptr;    // [eh][ew] sum of the row's weights before the texel
     double* env_rowsum = nullptr;    // [eh]
     double* env_total = nullptr;     // [1]
     int32_t* env_ok = nullptr;       // [1]
     uint32_t* env_marg = nullptr;    // [eh+1]
     uint32_t* env_cond = nullptr;    // [eh][ew+1]
     float4* env_texel = nullptr;     // [eh][ew]
-    uint32_t* env_gmarg = nullptr;   // [gm+1]
-    uint32_t* env_gcond = nullptr;   // [eh][gc+1]
     float4* env_row = nullptr;       // [eh]: (cos, sin of the row centre, RIS weight factor, 0)
     float2* env_col = nullptr;       // [ew]: (cos, sin of the column centre angle)
-    int gm_shift = 0, gc_shift = 0, gm = 1, gc = 1;
     // the CDF over all texels (row-major) that the draw inverts: 53-bit thresholds, its guide
     // and the FP64 sums of the rows before each row
     unsigned long long* env_flat = nullptr;  // [eh ew + 1] ceil(cdf 2^53)
