@@ -331,7 +331,7 @@ extern "C" mirres_status mirres_bvh_build(mirres_scene* s, void* stream)
     const cudaStream_t st = as_stream(stream);
     MR_TRY(mr_bvh_build(s, st));
     MR_TRY(mr_env_build(s, st));
-    s->ctx->host_launches += 20;
+    s->ctx->host_launches += 21;
     s->built = true;
     return MIRRES_OK;
 }
@@ -347,7 +347,7 @@ extern "C" mirres_status mirres_bvh_refit(mirres_scene* s, void* stream)
     const cudaStream_t st = as_stream(stream);
     MR_TRY(mr_bvh_refit(s, st));
     MR_TRY(mr_env_build(s, st));
-    s->ctx->host_launches += 6;
+    s->ctx->host_launches += 7;
     return MIRRES_OK;
 }
 

@@ -5,8 +5,8 @@
 //         stable LSD radix sort of the codes with the triangle id as payload (the initial
 //         order is by id, so the result is sorted by key = code << 32 | id) -> Karras's
 //         per-node hierarchy construction -> bottom-up boxes with arrival counters, which
-//         also writes the traversal layout (both child boxes in the parent, 64 bytes) and
-//         the packed triangles (v0, e1, e2; 48 bytes) in leaf order.
+//         also writes the packed triangles (v0, e1, e2; 48 bytes) in leaf order -> the traversal
+//         layout (both child boxes in the parent, 64 bytes, depth-first).
 //         With the PLOC builder selected the Karras step is replaced by locally-ordered
 //         clustering over the same Morton-sorted leaves (a lower-SAH tree, same layout).
 // refit:  bounds (vertex box only) -> bottom-up boxes, topology kept.
@@ -30,38 +30,42 @@ __device__ __forceinline__ float o2f(unsigned int u)
     return __uint_as_float((u & 0x80000000u) ? (u & 0x7fffffffu) : ~u);
 }
 
-// bounds[0..2] centroid lo, [3..5] centroid hi, [6..8] vertex lo, [9..11] vertex hi
-__global__ void k_init_bounds(unsigned int* bounds, int32_t* bad)
+// bounds[0..2] centroid lo, [3..5] centroid hi, [6..8] vertex lo, [9..11] vertex hi, each as the
+// ordered-integer image of the float, complemented for the lows so that all twelve are maxima and
+// zero bytes are their start; bounds[12] counts the blocks that are done.
+constexpr int BOUNDS_WORDS = 13;
+__device__ __forceinline__ bool bound_is_lo(int k) { return k < 3 || (k >= 6 && k < 9); }
+__device__ __forceinline__ float bound_of(const unsigned int* bounds, int k)
 {
-    const int i = threadIdx.x;
-    if (i < 12) {
-        const bool is_lo = (i < 3) || (i >= 6 && i < 9);
-        bounds[i] = is_lo ? f2o(__int_as_float(0x7f800000)) : f2o(__int_as_float(0xff800000));
-    }
-    if (i == 0) *bad = 0;
+    return o2f(bound_is_lo(k) ? ~bounds[k] : bounds[k]);
 }
 
-__device__ __forceinline__ int checked_index(const int32_t* tris, size_t k, int V, int32_t* bad)
+// a vertex index; an out-of-range one reads as vertex 0
+__device__ __forceinline__ int safe_index(const int32_t* tris, size_t k, int V)
 {
     const int i = __ldg(tris + k);
-    if (i < 0 || i >= V) {
-        *bad = 1;
-        return 0;
-    }
-    return i;
+    return (i < 0 || i >= V) ? 0 : i;
 }
 
+// Centroids, their box and the vertex box; the last block writes tmin. Bound by the gather of the
+// vertices; a block folds its twelve extrema in shared memory and issues one atomic each. (One
+// atomic per warp and extremum queued up at twelve addresses: 119 us for 499k triangles, now
+// 10.)
 __global__ void __launch_bounds__(256) k_bounds(const float* __restrict__ verts, const int32_t* __restrict__ tris,
                                                 int F, int V, float* __restrict__ cent, unsigned int* bounds,
-                                                int32_t* bad, int with_centroids)
+                                                float* tmin, int with_centroids)
 {
+    __shared__ unsigned int sb[12];
+    __shared__ bool last;
     const float INF = __int_as_float(0x7f800000);
     float b[12] = {INF, INF, INF, -INF, -INF, -INF, INF, INF, INF, -INF, -INF, -INF};
     const float third = 1.0f / 3.0f;
+    if (threadIdx.x < 12) sb[threadIdx.x] = 0u;
+    __syncthreads();
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < F; t += gridDim.x * blockDim.x) {
-        const int i0 = checked_index(tris, 3 * (size_t)t, V, bad);
-        const int i1 = checked_index(tris, 3 * (size_t)t + 1, V, bad);
-        const int i2 = checked_index(tris, 3 * (size_t)t + 2, V, bad);
+        const int i0 = safe_index(tris, 3 * (size_t)t, V);
+        const int i1 = safe_index(tris, 3 * (size_t)t + 1, V);
+        const int i2 = safe_index(tris, 3 * (size_t)t + 2, V);
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             const float a = __ldg(verts + 3 * (size_t)i0 + k), c1 = __ldg(verts + 3 * (size_t)i1 + k),
@@ -79,17 +83,26 @@ __global__ void __launch_bounds__(256) k_bounds(const float* __restrict__ verts,
     }
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
-        float v = b[k];
-        const bool is_lo = (k < 3) || (k >= 6 && k < 9);
-        for (int off = 16; off > 0; off >>= 1) {
-            const float o = __shfl_xor_sync(MR_FULL, v, off);
-            v = is_lo ? fminf(v, o) : fmaxf(v, o);
-        }
-        if ((threadIdx.x & 31) == 0) {
-            if (is_lo) atomicMin(bounds + k, f2o(v));
-            else atomicMax(bounds + k, f2o(v));
-        }
+        const unsigned int o = f2o(b[k]);
+        const unsigned int m = __reduce_max_sync(MR_FULL, bound_is_lo(k) ? ~o : o);
+        if ((threadIdx.x & 31) == 0) atomicMax(&sb[k], m);
     }
+    __syncthreads();
+    if (threadIdx.x < 12) {
+        atomicMax(bounds + threadIdx.x, sb[threadIdx.x]);
+        __threadfence();
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(bounds + 12, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last || threadIdx.x != 0) return;
+    __threadfence();
+    float e[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k)
+        e[k] = o2f(__ldcg(bounds + 9 + k)) - o2f(~__ldcg(bounds + 6 + k));
+    const float dx = e[0], dy = e[1], dz = e[2];
+    *tmin = F > 0 ? 1e-5f * sqrtf(dx * dx + dy * dy + dz * dz) : 0.0f;
 }
 
 __global__ void __launch_bounds__(256) k_check_indices(const int32_t* __restrict__ tris, int64_t n, int V,
@@ -101,19 +114,6 @@ __global__ void __launch_bounds__(256) k_check_indices(const int32_t* __restrict
         b = b || i < 0 || i >= V;
     }
     if (__any_sync(MR_FULL, b) && (threadIdx.x & 31) == 0) *bad = 1;
-}
-
-__global__ void k_finish_bounds(const unsigned int* bounds, int F, float* tmin)
-{
-    if (threadIdx.x != 0) return;
-    if (F <= 0) {
-        *tmin = 0.0f;
-        return;
-    }
-    const float dx = o2f(bounds[9]) - o2f(bounds[6]);
-    const float dy = o2f(bounds[10]) - o2f(bounds[7]);
-    const float dz = o2f(bounds[11]) - o2f(bounds[8]);
-    *tmin = 1e-5f * sqrtf(dx * dx + dy * dy + dz * dz);
 }
 
 __device__ __forceinline__ uint32_t expand10(uint32_t x)
@@ -133,7 +133,7 @@ __global__ void k_morton(const float* __restrict__ cent, const unsigned int* __r
     uint32_t q[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        const float lo = o2f(bounds[k]), hi = o2f(bounds[3 + k]);
+        const float lo = bound_of(bounds, k), hi = bound_of(bounds, 3 + k);
         const float ext = __fsub_rn(hi, lo);
         float f = 0.0f;
         if (ext > 0.0f) f = __fmul_rn(__fdiv_rn(__fsub_rn(cent[(size_t)k * F + t], lo), ext), 1024.0f);
@@ -162,51 +162,63 @@ __global__ void __launch_bounds__(RS_THREADS) k_rs_hist(const uint32_t* __restri
     hist[(size_t)threadIdx.x * nb + blockIdx.x] = h[threadIdx.x];
 }
 
-// exclusive scan of `total` entries in place, one block of 1024 threads
-__global__ void __launch_bounds__(1024) k_rs_scan(uint32_t* __restrict__ a, int total)
+// exclusive scan over a block of RS_THREADS; *total = the block's sum
+__device__ __forceinline__ uint32_t rs_block_scan(uint32_t v, uint32_t* total)
 {
-    __shared__ uint32_t wsum[32];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int seg = (total + 1023) / 1024;
-    const int start = tid * seg, end = min(start + seg, total);
-    uint32_t s = 0;
-    for (int i = start; i < end; ++i) s += a[i];
-    // inclusive scan of the per-thread sums
-    uint32_t x = s;
+    __shared__ uint32_t wsum[RS_THREADS / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    uint32_t x = v;
     for (int off = 1; off < 32; off <<= 1) {
         const uint32_t y = __shfl_up_sync(MR_FULL, x, off);
         if (lane >= off) x += y;
     }
     if (lane == 31) wsum[warp] = x;
     __syncthreads();
-    if (warp == 0) {
-        uint32_t w = wsum[lane];
-        for (int off = 1; off < 32; off <<= 1) {
-            const uint32_t y = __shfl_up_sync(MR_FULL, w, off);
-            if (lane >= off) w += y;
-        }
-        wsum[lane] = w;
+    uint32_t before = 0, all = 0;
+#pragma unroll
+    for (int w = 0; w < RS_THREADS / 32; ++w) {
+        if (w < warp) before += wsum[w];
+        all += wsum[w];
     }
-    __syncthreads();
-    uint32_t run = x - s + (warp > 0 ? wsum[warp - 1] : 0u);
-    for (int i = start; i < end; ++i) {
-        const uint32_t v = a[i];
-        a[i] = run;
-        run += v;
-    }
+    __syncthreads();  // (wsum is free for the next call)
+    *total = all;
+    return before + x - v;
 }
 
+// Block d: exclusive scan of digit d's counts over the tiles, in place, and their sum. (A single
+// block scanned all 256 nb counts, each thread a strided segment: 47 us a pass at 499k triangles,
+// now 2.)
+__global__ void __launch_bounds__(RS_THREADS) k_rs_scan(uint32_t* __restrict__ hist, int nb, uint32_t* __restrict__ sum)
+{
+    uint32_t* const a = hist + (size_t)blockIdx.x * nb;
+    uint32_t run = 0;
+    for (int base = 0; base < nb; base += RS_THREADS) {  // block-uniform
+        const int i = base + (int)threadIdx.x;
+        uint32_t total;
+        const uint32_t e = rs_block_scan(i < nb ? a[i] : 0u, &total);
+        if (i < nb) a[i] = run + e;
+        run += total;
+    }
+    if (threadIdx.x == 0) sum[blockIdx.x] = run;
+}
+
+// LAST: the sorted order goes out as the keys code << 32 | triangle and the leaf order
+template <bool LAST>
 __global__ void __launch_bounds__(RS_THREADS) k_rs_scatter(const uint32_t* __restrict__ kin,
                                                            const int32_t* __restrict__ vin,
                                                            uint32_t* __restrict__ kout, int32_t* __restrict__ vout,
                                                            int n, int shift, const uint32_t* __restrict__ offs,
-                                                           int nb)
+                                                           const uint32_t* __restrict__ sum, int nb,
+                                                           uint64_t* __restrict__ keys)
 {
     constexpr int NW = RS_THREADS / 32;
     __shared__ uint32_t base[256];
     __shared__ uint32_t wcnt[NW][256];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    base[tid] = offs[(size_t)tid * nb + blockIdx.x];
+    static_assert(RS_THREADS == 256, "one thread per digit");
+    uint32_t all;
+    const uint32_t digit_base = rs_block_scan(sum[tid], &all);
+    base[tid] = digit_base + offs[(size_t)tid * nb + blockIdx.x];
 #pragma unroll
     for (int w = 0; w < NW; ++w) wcnt[w][tid] = 0;
     __syncthreads();
@@ -231,7 +243,8 @@ __global__ void __launch_bounds__(RS_THREADS) k_rs_scatter(const uint32_t* __res
         __syncthreads();
         if (valid) {
             const uint32_t dst = base[dig] + wcnt[warp][dig] + (uint32_t)rank;
-            kout[dst] = k;
+            if (LAST) keys[dst] = ((uint64_t)k << 32) | (uint32_t)v;
+            else kout[dst] = k;
             vout[dst] = v;
         }
         __syncthreads();
@@ -242,15 +255,6 @@ __global__ void __launch_bounds__(RS_THREADS) k_rs_scatter(const uint32_t* __res
     }
 }
 
-__global__ void k_keys(const uint32_t* __restrict__ codes, const int32_t* __restrict__ vals, int F,
-                       uint64_t* __restrict__ keys, int32_t* __restrict__ perm)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= F) return;
-    keys[i] = ((uint64_t)codes[i] << 32) | (uint32_t)vals[i];
-    perm[i] = vals[i];
-}
-
 // ---- Karras 2012 hierarchy: one thread per internal node ---------------------------------
 __device__ __forceinline__ int delta(const uint64_t* __restrict__ k, int F, int i, int j)
 {
@@ -259,7 +263,7 @@ __device__ __forceinline__ int delta(const uint64_t* __restrict__ k, int F, int 
 }
 
 __global__ void k_karras(const uint64_t* __restrict__ k, int F, int32_t* __restrict__ left,
-                         int32_t* __restrict__ right, int32_t* __restrict__ parent)
+                         int32_t* __restrict__ right, int32_t* __restrict__ parent, int2* __restrict__ range)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= F - 1) return;
@@ -281,6 +285,7 @@ __global__ void k_karras(const uint64_t* __restrict__ k, int F, int32_t* __restr
     }
     const int g = i + s * d + min(d, 0);
     const int lo = min(i, j), hi = max(i, j);
+    range[i] = make_int2(lo, hi - lo + 1);  // first leaf position, leaf count
     if (lo == g) {
         left[i] = ~g;
         parent[(F - 1) + g] = i;
@@ -297,70 +302,139 @@ __global__ void k_karras(const uint64_t* __restrict__ k, int F, int32_t* __restr
     }
 }
 
-// ---- bottom-up boxes, traversal layout, packed triangles ---------------------------------
-__global__ void k_bottom_up(const float* __restrict__ verts, const int32_t* __restrict__ tris, int F, int V,
-                            const int32_t* __restrict__ perm, const int32_t* __restrict__ left,
-                            const int32_t* __restrict__ right, const int32_t* __restrict__ parent,
-                            float* lo, float* hi, int32_t* flags, float4* __restrict__ nodes,
-                            float4* __restrict__ ptri, int32_t* __restrict__ leaf_of, int2* __restrict__ range)
+// ---- bottom-up boxes, packed triangles ----------------------------------------------------
+// One thread per leaf climbs while it is the second to arrive, carrying the box of the subtree it
+// finished in registers; the first arriver leaves its box in its half of the parent's node record
+// for the other. Through global memory that exchange (store, fence, atomic, load) costs L2 round
+// trips on every level, and these bound the kernel. KARRAS: a node's leaves are a contiguous range
+// that holds the node's own id, so a node whose range lies within a block's 256 leaves is finished
+// by that block alone, through shared memory: all but ~1/256 of the nodes, and about eight of the
+// levels on a leaf's path. Only the rest goes through L2, as all of it does for a clustering tree
+// (whose ids and ranges say nothing; its leaf counts are taken on the way). 499k triangles: 128 us
+// with every level through L2 and both children's boxes read back with twelve 4-byte loads, now
+// 65.
+constexpr int BU_BLOCK = 256;
+
+// a box as three pairs: (min.xy) (min.z, max.x) (max.yz)
+struct Box6 {
+    float2 a, b, c;
+};
+__device__ __forceinline__ Box6 box_union(const Box6& x, const Box6& y)
 {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    return Box6{make_float2(fminf(x.a.x, y.a.x), fminf(x.a.y, y.a.y)), make_float2(fminf(x.b.x, y.b.x), fmaxf(x.b.y, y.b.y)),
+                make_float2(fmaxf(x.c.x, y.c.x), fmaxf(x.c.y, y.c.y))};
+}
+__device__ __forceinline__ void box_export(const Box6& x, float* lo, float* hi, size_t n)
+{
+    lo[3 * n] = x.a.x;
+    lo[3 * n + 1] = x.a.y;
+    lo[3 * n + 2] = x.b.x;
+    hi[3 * n] = x.b.y;
+    hi[3 * n + 1] = x.c.x;
+    hi[3 * n + 2] = x.c.y;
+}
+
+// counts an arrival at a node (acquire and release at GPU scope: what either arriver stored before
+// it is visible to the second); returns the arrivals before it
+__device__ __forceinline__ int arrive(int32_t* flag)
+{
+    int old;
+    asm volatile("atom.add.acq_rel.gpu.global.s32 %0, [%1], 1;" : "=r"(old) : "l"(flag) : "memory");
+    return old;
+}
+
+template <bool KARRAS>
+__global__ void __launch_bounds__(BU_BLOCK) k_bottom_up(const float* __restrict__ verts, const int32_t* __restrict__ tris,
+                                                        int F, int V, const int32_t* __restrict__ perm,
+                                                        const int32_t* __restrict__ left,
+                                                        const int32_t* __restrict__ right,
+                                                        const int32_t* __restrict__ parent, float* __restrict__ lo,
+                                                        float* __restrict__ hi, int32_t* flags, float2* nodes,
+                                                        float4* __restrict__ ptri, int32_t* __restrict__ leaf_of,
+                                                        int2* range)
+{
+    __shared__ Box6 half[KARRAS ? 2 * BU_BLOCK : 1];  // by node id - b0, left and right child
+    __shared__ int arrived[KARRAS ? BU_BLOCK : 1];
+    __shared__ int2 up[KARRAS ? BU_BLOCK : 1];  // of a node inside the block: its parent, whether it is the
+                                                // right child there; (-2, -) otherwise
+    const int b0 = blockIdx.x * BU_BLOCK, j = b0 + (int)threadIdx.x;
+    if (KARRAS) {
+        int2 u = make_int2(-2, 0);
+        if (j < F - 1) {
+            const int2 r = range[j];
+            if (r.x >= b0 && r.x + r.y <= b0 + BU_BLOCK) {
+                const int up_id = parent[j];
+                u = make_int2(up_id, up_id >= 0 && right[up_id] == j);
+            }
+        }
+        up[threadIdx.x] = u;
+        arrived[threadIdx.x] = 0;
+        __syncthreads();
+    }
     if (j >= F) return;
     const int t = perm[j];
-    int idx[3];
+    float3 q[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-        const int v = __ldg(tris + 3 * (size_t)t + c);
-        idx[c] = (v >= 0 && v < V) ? v : 0;
+        const int v = safe_index(tris, 3 * (size_t)t + c, V);
+        q[c] = f3(verts[3 * (size_t)v], verts[3 * (size_t)v + 1], verts[3 * (size_t)v + 2]);
     }
-    const float3 a = f3(verts[3 * (size_t)idx[0]], verts[3 * (size_t)idx[0] + 1], verts[3 * (size_t)idx[0] + 2]);
-    const float3 b = f3(verts[3 * (size_t)idx[1]], verts[3 * (size_t)idx[1] + 1], verts[3 * (size_t)idx[1] + 2]);
-    const float3 c = f3(verts[3 * (size_t)idx[2]], verts[3 * (size_t)idx[2] + 1], verts[3 * (size_t)idx[2] + 2]);
+    const float3 a = q[0], b = q[1], c = q[2];
+    Box6 x{make_float2(fminf(fminf(a.x, b.x), c.x), fminf(fminf(a.y, b.y), c.y)),
+           make_float2(fminf(fminf(a.z, b.z), c.z), fmaxf(fmaxf(a.x, b.x), c.x)),
+           make_float2(fmaxf(fmaxf(a.y, b.y), c.y), fmaxf(fmaxf(a.z, b.z), c.z))};
     const size_t L = (size_t)(F - 1) + j;
-    lo[3 * L] = fminf(fminf(a.x, b.x), c.x);
-    lo[3 * L + 1] = fminf(fminf(a.y, b.y), c.y);
-    lo[3 * L + 2] = fminf(fminf(a.z, b.z), c.z);
-    hi[3 * L] = fmaxf(fmaxf(a.x, b.x), c.x);
-    hi[3 * L + 1] = fmaxf(fmaxf(a.y, b.y), c.y);
-    hi[3 * L + 2] = fmaxf(fmaxf(a.z, b.z), c.z);
+    box_export(x, lo, hi, L);
     float4* pt = ptri + MR_TRI_STRIDE * (size_t)j;
     pt[0] = make_float4(a.x, a.y, a.z, __int_as_float(t));
     pt[1] = make_float4(b.x - a.x, b.y - a.y, b.z - a.z, 0.0f);
     pt[2] = make_float4(c.x - a.x, c.y - a.y, c.z - a.z, 0.0f);
     if (MR_TRI_STRIDE == 4) pt[3] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     leaf_of[t] = j;
+    int2 rg = make_int2(j, 1);  // clustering trees: (least leaf position, leaf count) so far
     int p = parent[L];
+    bool is_right = p >= 0 && right[p] == ~j;
     while (p >= 0) {
-        __threadfence();
-        if (atomicAdd(&flags[p], 1) == 0) return;  // the sibling's thread finishes this node
-        __threadfence();
-        const int cl = left[p], cr = right[p];
-        const size_t il = cl >= 0 ? (size_t)cl : (size_t)(F - 1) + ~cl;
-        const size_t ir = cr >= 0 ? (size_t)cr : (size_t)(F - 1) + ~cr;
-        float bl[6], br[6];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            bl[k] = __ldcg(lo + 3 * il + k);
-            bl[3 + k] = __ldcg(hi + 3 * il + k);
-            br[k] = __ldcg(lo + 3 * ir + k);
-            br[3 + k] = __ldcg(hi + 3 * ir + k);
+        const int n = KARRAS ? p - b0 : 0;
+        const int2 u = (KARRAS && n >= 0 && n < BU_BLOCK) ? up[n] : make_int2(-2, 0);
+        float2* const rec = nodes + 6 * (size_t)p;  // left box, right box
+        float2* const mine = rec + (is_right ? 3 : 0);
+        float2* const other = rec + (is_right ? 0 : 3);
+        Box6 o;
+        int next;
+        bool next_right;
+        if (u.x != -2) {  // inside the block: the exchange stays in shared memory
+            half[2 * n + (is_right ? 1 : 0)] = x;
+            __threadfence_block();
+            if (atomicAdd(&arrived[n], 1) == 0) return;  // the sibling's thread finishes this node
+            __threadfence_block();
+            o = half[2 * n + (is_right ? 0 : 1)];
+            other[0] = o.a;
+            other[1] = o.b;
+            other[2] = o.c;
+            mine[0] = x.a;
+            mine[1] = x.b;
+            mine[2] = x.c;
+            next = u.x;
+            next_right = u.y != 0;
+        } else {
+            __stcg(mine, x.a);
+            __stcg(mine + 1, x.b);
+            __stcg(mine + 2, x.c);
+            next = parent[p];  // (on their way while the stores are)
+            next_right = next >= 0 && right[next] == p;
+            if (arrive(&flags[p]) == 0) return;
+            o = Box6{__ldcg(other), __ldcg(other + 1), __ldcg(other + 2)};
         }
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            __stcg(lo + 3 * (size_t)p + k, fminf(bl[k], br[k]));
-            __stcg(hi + 3 * (size_t)p + k, fmaxf(bl[3 + k], br[3 + k]));
+        x = box_union(x, o);
+        if (!KARRAS) {
+            const int sib = is_right ? left[p] : right[p];
+            const int2 rs = sib >= 0 ? __ldcg(range + sib) : make_int2(~sib, 1);
+            rg = make_int2(min(rg.x, rs.x), rg.y + rs.y);
+            __stcg(range + p, rg);
         }
-        nodes[4 * (size_t)p] = make_float4(bl[0], bl[1], bl[2], bl[3]);
-        nodes[4 * (size_t)p + 1] = make_float4(bl[4], bl[5], br[0], br[1]);
-        nodes[4 * (size_t)p + 2] = make_float4(br[2], br[3], br[4], br[5]);
-        nodes[4 * (size_t)p + 3] = make_float4(__int_as_float(cl), __int_as_float(cr), 0.0f, 0.0f);
-        // (first leaf position, leaf count) under p: the count is exact for every builder, the
-        // first position delimits the subtree only for the Karras tree (clustering may pair
-        // clusters that are not neighbours)
-        const int2 rl = cl >= 0 ? __ldcg(range + cl) : make_int2(~cl, 1);
-        const int2 rr = cr >= 0 ? __ldcg(range + cr) : make_int2(~cr, 1);
-        __stcg(range + p, make_int2(min(rl.x, rr.x), rl.y + rr.y));
-        p = parent[p];
+        p = next;
+        is_right = next_right;
     }
 }
 
@@ -370,39 +444,42 @@ __global__ void k_bottom_up(const float* __restrict__ verts, const int32_t* __re
 // the ones it just read, and every subtree is one contiguous block. Preorder position of a node:
 // its parent's plus 1 when it is the left child, plus 1 + (internal nodes of the left sibling's
 // subtree) = the left sibling's leaf count (1 for a leaf) when it is the right child; each
-// thread sums these up its path to the root. The boxes are copied unchanged, the children's
-// node ids mapped to their positions (leaf children keep their leaf positions).
-__global__ void k_dfs_index(const int32_t* __restrict__ parent, const int32_t* __restrict__ left,
-                            const int2* __restrict__ range, int F, int32_t* __restrict__ dfs)
+// thread sums these up its path to the root and copies its node there; its children's positions
+// follow from its own by the same rule (leaf children keep their leaf positions). It also writes
+// the node's own box, the union of its children's, to the export arrays.
+template <bool KARRAS>
+__global__ void __launch_bounds__(256) k_dfs_nodes(const int32_t* __restrict__ parent, const int32_t* __restrict__ left,
+                                                   const int32_t* __restrict__ right, const int2* __restrict__ range,
+                                                   const float4* __restrict__ nodes, int F, float4* __restrict__ dnodes,
+                                                   float* __restrict__ lo, float* __restrict__ hi)
 {
     const int n = blockIdx.x * blockDim.x + threadIdx.x;
     if (n >= F - 1) return;
-    int idx = 0, c = n;
+    const float4 n0 = nodes[3 * (size_t)n], n1 = nodes[3 * (size_t)n + 1], n2 = nodes[3 * (size_t)n + 2];
+    const Box6 bl{make_float2(n0.x, n0.y), make_float2(n0.z, n0.w), make_float2(n1.x, n1.y)};
+    const Box6 br{make_float2(n1.z, n1.w), make_float2(n2.x, n2.y), make_float2(n2.z, n2.w)};
+    box_export(box_union(bl, br), lo, hi, (size_t)n);
+    int q = 0, c = n;
     for (int depth = 0; c != 0 && depth < 2 * F; ++depth) {  // every kept tree is at most 64 deep
         const int p = parent[c];
         if (p < 0) break;
         const int l = left[p];
-        idx += (l == c) ? 1 : (l >= 0 ? range[l].y : 1);
+        // (the leaves of all left siblings on the way are those before the node's first leaf)
+        if (KARRAS) q += (l == c) ? 1 : 0;
+        else q += (l == c) ? 1 : (l >= 0 ? range[l].y : 1);
         c = p;
     }
-    dfs[n] = idx;
-}
-
-__global__ void k_dfs_gather(const float4* __restrict__ nodes, const int32_t* __restrict__ dfs, int F,
-                             float4* __restrict__ dnodes)
-{
-    const int n = blockIdx.x * blockDim.x + threadIdx.x;
-    if (n >= F - 1) return;
-    const int q = dfs[n];
+    if (KARRAS) q += range[n].x;
     if (q < 0 || q >= F - 1) return;  // (not for a well-formed tree: its positions are a permutation)
-    dnodes[4 * (size_t)q] = nodes[4 * (size_t)n];
-    dnodes[4 * (size_t)q + 1] = nodes[4 * (size_t)n + 1];
-    dnodes[4 * (size_t)q + 2] = nodes[4 * (size_t)n + 2];
-    const float4 ch = nodes[4 * (size_t)n + 3];
-    int cl = __float_as_int(ch.x), cr = __float_as_int(ch.y);
-    if (cl >= 0) cl = dfs[cl];
-    if (cr >= 0) cr = dfs[cr];
-    dnodes[4 * (size_t)q + 3] = make_float4(__int_as_float(cl), __int_as_float(cr), 0.0f, 0.0f);
+    int cl = left[n], cr = right[n];
+    const int leaves = cl >= 0 ? range[cl].y : 1;
+    if (cl >= 0) cl = q + 1;
+    if (cr >= 0) cr = q + leaves;
+    float4* const dst = dnodes + 4 * (size_t)q;
+    dst[0] = n0;
+    dst[1] = n1;
+    dst[2] = n2;
+    dst[3] = make_float4(__int_as_float(cl), __int_as_float(cr), 0.0f, 0.0f);
 }
 
 // ---- PLOC hierarchy: parallel locally-ordered clustering (Meister and Bittner 2018) ------
@@ -747,9 +824,8 @@ mirres_status mr_bvh_alloc(mirres_scene* s)
     MR_TRY(mr_alloc(&s->lo, 3 * (F > 0 ? 2 * F - 1 : 1)));
     MR_TRY(mr_alloc(&s->hi, 3 * (F > 0 ? 2 * F - 1 : 1)));
     MR_TRY(mr_alloc(&s->flags, F > 1 ? F - 1 : 1));
-    MR_TRY(mr_alloc(&s->nodes, 4 * (F > 1 ? F - 1 : 1)));
+    MR_TRY(mr_alloc(&s->nodes, 3 * (F > 1 ? F - 1 : 1)));
     MR_TRY(mr_alloc(&s->dnodes, 4 * (F > 1 ? F - 1 : 1)));
-    MR_TRY(mr_alloc(&s->dfs, F > 1 ? F - 1 : 1));
     MR_TRY(mr_alloc(&s->ptri, MR_TRI_STRIDE * F));
     MR_TRY(mr_alloc(&s->leaf_of, F));
     MR_TRY(mr_alloc(&s->range, F > 1 ? F - 1 : 1));
@@ -758,8 +834,8 @@ mirres_status mr_bvh_alloc(mirres_scene* s)
     MR_TRY(mr_alloc(&s->codes[1], F));
     MR_TRY(mr_alloc(&s->vals[0], F));
     MR_TRY(mr_alloc(&s->vals[1], F));
-    MR_TRY(mr_alloc(&s->hist, 256 * (nb ? nb : 1)));
-    MR_TRY(mr_alloc(&s->bounds, 12));
+    MR_TRY(mr_alloc(&s->hist, 256 * (nb ? nb : 1) + 256));
+    MR_TRY(mr_alloc(&s->bounds, BOUNDS_WORDS));
     MR_TRY(mr_alloc(&s->tmin, 1));
     MR_TRY(mr_alloc(&s->bad, 1));
     return MIRRES_OK;
@@ -770,7 +846,7 @@ void mr_bvh_free(mirres_scene* s)
     void* ptrs[] = {s->keys, s->perm, s->left, s->right, s->parent, s->lo, s->hi, s->flags, s->nodes, s->ptri,
                     s->leaf_of, s->cent, s->codes[0], s->codes[1], s->vals[0], s->vals[1], s->hist, s->bounds,
                     s->tmin, s->bad, s->ploc_box, s->ploc_node, s->ploc_nn, s->ploc_part, s->ploc_state,
-                    s->vacc, s->vnrm, s->gvn, s->range, s->dnodes, s->dfs};
+                    s->vacc, s->vnrm, s->gvn, s->range, s->dnodes};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     mr_wide_free(s);
@@ -781,13 +857,12 @@ static mirres_status bottom_up(mirres_scene* s, cudaStream_t st)
     const int F = s->desc.n_tris;
     if (F <= 0) return MIRRES_OK;
     if (F > 1) MR_CUDA(cudaMemsetAsync(s->flags, 0, sizeof(int32_t) * (size_t)(F - 1), st));
-    k_bottom_up<<<grid_for(F, 256), 256, 0, st>>>(s->desc.verts, s->desc.tris, F, s->desc.n_verts, s->perm, s->left,
-                                                 s->right, s->parent, s->lo, s->hi, s->flags, s->nodes, s->ptri,
-                                                 s->leaf_of, s->range);
-    if (F > 1) {
-        k_dfs_index<<<grid_for(F - 1, 256), 256, 0, st>>>(s->parent, s->left, s->range, F, s->dfs);
-        k_dfs_gather<<<grid_for(F - 1, 256), 256, 0, st>>>(s->nodes, s->dfs, F, s->dnodes);
-    }
+    (s->karras ? k_bottom_up<true> : k_bottom_up<false>)<<<grid_for(F, BU_BLOCK), BU_BLOCK, 0, st>>>(
+        s->desc.verts, s->desc.tris, F, s->desc.n_verts, s->perm, s->left, s->right, s->parent, s->lo, s->hi, s->flags,
+        reinterpret_cast<float2*>(s->nodes), s->ptri, s->leaf_of, s->range);
+    if (F > 1)
+        (s->karras ? k_dfs_nodes<true> : k_dfs_nodes<false>)<<<grid_for(F - 1, 256), 256, 0, st>>>(
+            s->parent, s->left, s->right, s->range, s->nodes, F, s->dnodes, s->lo, s->hi);
     MR_CUDA(cudaGetLastError());
     return MIRRES_OK;
 }
@@ -795,14 +870,9 @@ static mirres_status bottom_up(mirres_scene* s, cudaStream_t st)
 static mirres_status bounds(mirres_scene* s, cudaStream_t st, int with_centroids)
 {
     const int F = s->desc.n_tris;
-    k_init_bounds<<<1, 32, 0, st>>>(s->bounds, s->bad);
-    if (F > 0) {
-        int grid = grid_for(F, 256);
-        if (grid > 4096) grid = 4096;
-        k_bounds<<<grid, 256, 0, st>>>(s->desc.verts, s->desc.tris, F, s->desc.n_verts, s->cent, s->bounds, s->bad,
-                                       with_centroids);
-    }
-    k_finish_bounds<<<1, 32, 0, st>>>(s->bounds, F, s->tmin);
+    MR_CUDA(cudaMemsetAsync(s->bounds, 0, sizeof(unsigned int) * BOUNDS_WORDS, st));
+    k_bounds<<<std::min(std::max(grid_for(F, 256), 1), s->ctx->sm_count * 4), 256, 0, st>>>(
+        s->desc.verts, s->desc.tris, F, s->desc.n_verts, s->cent, s->bounds, s->tmin, with_centroids);
     MR_CUDA(cudaGetLastError());
     return MIRRES_OK;
 }
@@ -879,15 +949,17 @@ mirres_status mr_bvh_build(mirres_scene* s, cudaStream_t st)
     if (F > 0) {
         const int nb = (F + RS_TILE - 1) / RS_TILE;
         k_morton<<<grid_for(F, 256), 256, 0, st>>>(s->cent, s->bounds, F, s->codes[0], s->vals[0]);
+        uint32_t* const sum = s->hist + (size_t)256 * nb;  // [256] digit totals behind the tile counts
         int cur = 0;
         for (int shift = 0; shift < 32; shift += 8) {
             k_rs_hist<<<nb, RS_THREADS, 0, st>>>(s->codes[cur], F, shift, s->hist, nb);
-            k_rs_scan<<<1, 1024, 0, st>>>(s->hist, 256 * nb);
-            k_rs_scatter<<<nb, RS_THREADS, 0, st>>>(s->codes[cur], s->vals[cur], s->codes[cur ^ 1], s->vals[cur ^ 1],
-                                                    F, shift, s->hist, nb);
+            k_rs_scan<<<256, RS_THREADS, 0, st>>>(s->hist, nb, sum);
+            const bool last = shift == 24;
+            (last ? k_rs_scatter<true> : k_rs_scatter<false>)<<<nb, RS_THREADS, 0, st>>>(
+                s->codes[cur], s->vals[cur], s->codes[cur ^ 1], last ? s->perm : s->vals[cur ^ 1], F, shift, s->hist,
+                sum, nb, s->keys);
             cur ^= 1;
         }
-        k_keys<<<grid_for(F, 256), 256, 0, st>>>(s->codes[cur], s->vals[cur], F, s->keys, s->perm);
         MR_CUDA(cudaMemsetAsync(s->parent, 0xFF, sizeof(int32_t) * (size_t)(2 * F - 1), st));
         bool karras = F > 1;
         if (F > 1 && s->builder == MIRRES_BVH_PLOC) {
@@ -896,7 +968,8 @@ mirres_status mr_bvh_build(mirres_scene* s, cudaStream_t st)
             karras = too_deep;
             if (too_deep) MR_CUDA(cudaMemsetAsync(s->parent, 0xFF, sizeof(int32_t) * (size_t)(2 * F - 1), st));
         }
-        if (karras) k_karras<<<grid_for(F - 1, 256), 256, 0, st>>>(s->keys, F, s->left, s->right, s->parent);
+        if (karras) k_karras<<<grid_for(F - 1, 256), 256, 0, st>>>(s->keys, F, s->left, s->right, s->parent, s->range);
+        s->karras = karras;
         MR_CUDA(cudaGetLastError());
         MR_TRY(bottom_up(s, st));
         if (s->traversal == MIRRES_TRAVERSAL_WIDE) MR_TRY(mr_wide_build(s, st));

@@ -68,9 +68,9 @@ struct mirres_scene {
     float* lo = nullptr;             // [2F-1][3]
     float* hi = nullptr;             // [2F-1][3]
     int32_t* flags = nullptr;        // [F-1] bottom-up arrival counters
-    float4* nodes = nullptr;         // [F-1][4] by internal node id (the builders' layout)
-    float4* dnodes = nullptr;        // [F-1][4] the same nodes in depth-first preorder (traversal)
-    int32_t* dfs = nullptr;          // [F-1] internal node id -> its position in dnodes
+    float4* nodes = nullptr;         // [F-1][3] both child boxes by internal node id (the builders' order)
+    float4* dnodes = nullptr;        // [F-1][4] the traversal's nodes: child boxes and codes, depth-first preorder
+    bool karras = true;              // the hierarchy of the last build is the Karras tree (ids within their ranges)
     float4* ptri = nullptr;          // [F][3]
     int32_t* leaf_of = nullptr;      // [F]
     int2* range = nullptr;           // [F-1] (first leaf position, leaf count) under each internal node
@@ -82,8 +82,8 @@ struct mirres_scene {
     float* cent = nullptr;           // [3][F] centroids (build scratch)
     uint32_t* codes[2] = {nullptr, nullptr};
     int32_t* vals[2] = {nullptr, nullptr};
-    uint32_t* hist = nullptr;        // radix histograms
-    unsigned int* bounds = nullptr;  // [12] ordered-uint bounds: centroid lo/hi, vertex lo/hi
+    uint32_t* hist = nullptr;        // radix histograms and digit totals
+    unsigned int* bounds = nullptr;  // [13] ordered-uint bounds: centroid lo/hi, vertex lo/hi; blocks done
     float* tmin = nullptr;           // [1]
     int32_t* bad = nullptr;          // [1] invalid index flag
     // shading normals: MIRRES_NORMALS_FACE or MIRRES_NORMALS_INTERPOLATED (area-weighted vertex
