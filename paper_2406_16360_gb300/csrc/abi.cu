@@ -1368,18 +1368,18 @@ extern "C" mirres_status mirres_gbuffer(mirres_context* ctx, const mirres_scene*
     return MIRRES_OK;
 }
 
-// record layout (16-byte aligned) for a stack of n images of npx pixels: packed normals and
-// positions [n][H][W] float4, the levels' inputs c_i [levels][n][H][W] float4, their reciprocal
-// normalisers 1 / k_i [levels][n][H][W] float
+// record layout (16-byte aligned) for a stack of n images of npx pixels: the G-buffer
+// [n][H][W] (normal.xyz, position.x) (position.yz, -, -), the levels' inputs c_i [levels][n][H][W]
+// float4, their reciprocal normalisers 1 / k_i [levels][n][H][W] float
 struct EawtRecord {
-    float4 *n, *x, *c;
+    float4 *g, *c;
     float* ik;
 };
 
 static EawtRecord eawt_record(void* base, size_t npx, int L)
 {
     float4* f = reinterpret_cast<float4*>(base);
-    return EawtRecord{f, f + npx, f + 2 * npx, reinterpret_cast<float*>(f + (2 + (size_t)L) * npx)};
+    return EawtRecord{f, f + 2 * npx, reinterpret_cast<float*>(f + (2 + (size_t)L) * npx)};
 }
 
 static mirres_status eawt_args(int32_t n_images, int32_t width, int32_t height, const mirres_eawt_params* params,
@@ -1407,20 +1407,18 @@ extern "C" mirres_status mirres_eawt_batch(mirres_context* ctx, int32_t n_images
     const size_t npx = (size_t)width * height * n_images;
     const int L = params->levels, sms = ctx->sm_count;
     const EawtRecord r = eawt_record(record, npx, L);
-    mr_launch_eawt_pack(normal, r.n, (int64_t)npx, sms, st);
-    mr_launch_eawt_pack(position, r.x, (int64_t)npx, sms, st);
-    mr_launch_eawt_pack(image, r.c, (int64_t)npx, sms, st);
+    mr_launch_eawt_pack(image, normal, position, r.c, r.g, (int64_t)npx, sms, st);
     const float in2 = 1.0f / (params->sigma_n * params->sigma_n), ix2 = 1.0f / (params->sigma_x * params->sigma_x);
     for (int i = 0; i < L; ++i) {
         const int step = 1 << i;
         const float srt = params->sigma_rt / (float)step;
         const bool last = i + 1 == L;
-        mr_launch_eawt_level(r.c + npx * (size_t)i, r.n, r.x, n_images, width, height, step, 1.0f / (srt * srt), in2,
-                             ix2, last ? nullptr : r.c + npx * (size_t)(i + 1), last ? out : nullptr,
-                             r.ik + npx * (size_t)i, sms, st);
+        mr_launch_eawt_level(r.c + npx * (size_t)i, r.g, n_images, width, height, i, 1.0f / (srt * srt), in2, ix2,
+                             last ? nullptr : r.c + npx * (size_t)(i + 1), last ? out : nullptr,
+                             r.ik + npx * (size_t)i, st);
     }
     MR_CUDA(cudaGetLastError());
-    ctx->host_launches += (unsigned long long)L + 3;
+    ctx->host_launches += (unsigned long long)L + 1;
     return MIRRES_OK;
 }
 
@@ -1451,14 +1449,14 @@ extern "C" mirres_status mirres_eawt_batch_backward(mirres_context* ctx, int32_t
     float4* tmp[2] = {reinterpret_cast<float4*>(ctx->ws.ptr), reinterpret_cast<float4*>(ctx->ws.ptr) + npx};
     const EawtRecord r = eawt_record(const_cast<void*>(record), npx, L);
     const float in2 = 1.0f / (params->sigma_n * params->sigma_n), ix2 = 1.0f / (params->sigma_x * params->sigma_x);
-    mr_launch_eawt_pack(d_out, tmp[0], (int64_t)npx, sms, st);
+    mr_launch_eawt_pack_adjoint(d_out, r.ik + npx * (size_t)(L - 1), tmp[0], (int64_t)npx, sms, st);
     int cur = 0;
     for (int i = L - 1; i >= 0; --i) {
         const int step = 1 << i;
         const float srt = params->sigma_rt / (float)step;
-        mr_launch_eawt_level_adjoint(tmp[cur], r.c + npx * (size_t)i, r.ik + npx * (size_t)i, r.n, r.x, n_images,
-                                     width, height, step, 1.0f / (srt * srt), in2, ix2,
-                                     i == 0 ? nullptr : tmp[cur ^ 1], i == 0 ? d_image : nullptr, sms, st);
+        mr_launch_eawt_level_adjoint(tmp[cur], r.c + npx * (size_t)i, r.g, n_images, width, height, i,
+                                     1.0f / (srt * srt), in2, ix2, i == 0 ? nullptr : tmp[cur ^ 1],
+                                     i == 0 ? d_image : nullptr, i == 0 ? nullptr : r.ik + npx * (size_t)(i - 1), st);
         cur ^= 1;
     }
     MR_CUDA(cudaGetLastError());

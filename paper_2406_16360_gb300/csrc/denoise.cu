@@ -7,186 +7,164 @@
 // sigma_rt_i = sigma_rt / 2^i and k(p) = sum_q h w; taps outside the image are left out. The
 // adjoint holds the weights fixed: since h w(p, q) is symmetric in p and q, the transpose of a
 // level is the same stencil applied to g / k. Every launch covers a stack of images of one size.
+#include <algorithm>
+
 #include "render.h"
 
 namespace {
 
-__constant__ float kB3[5] = {1.0f / 16.0f, 4.0f / 16.0f, 6.0f / 16.0f, 4.0f / 16.0f, 1.0f / 16.0f};
+// log2 of the B3 taps (1, 4, 6, 4, 1) / 16: the tap's weight goes into the exponent
+__constant__ float kLogB3[5] = {-4.0f, -2.0f, -1.41503749927884381f, -2.0f, -4.0f};
+constexpr float kLog2e = 1.44269504088896341f;
 
-// The level kernels read packed float4 images (colour / normal / position in .xyz): one
-// 16-byte load per buffer and tap instead of three scalar loads.
-__global__ void __launch_bounds__(256) k_eawt_pack(const float* __restrict__ a, float4* __restrict__ out, int64_t npx)
+__device__ __forceinline__ float exp2_approx(float x)
 {
-    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < npx; p += (int64_t)gridDim.x * blockDim.x)
-        out[p] = make_float4(__ldg(a + 3 * p), __ldg(a + 3 * p + 1), __ldg(a + 3 * p + 2), 0.0f);
+    float r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
 }
 
-__device__ __forceinline__ float d2(float4 a, float4 b)
+// The level kernels read the colour as one float4 a pixel and the G-buffer as one 32-byte record
+// (normal.xyz, position.x) (position.yz, -, -): one 16-byte and one 32-byte load per tap (two of 16
+// bytes where the record is not 32-byte aligned: ALIGNED = false).
+struct Guide {
+    float nx, ny, nz, x, y, z;
+};
+template <bool ALIGNED>
+__device__ __forceinline__ Guide guide_at(const float4* __restrict__ g, uint32_t p)
 {
-    const float x = a.x - b.x, y = a.y - b.y, z = a.z - b.z;
-    return x * x + y * y + z * z;
-}
-
-__device__ __forceinline__ void store(float4* o4, float* o3, int64_t p, float x, float y, float z)
-{
-    if (o3) {
-        o3[3 * p] = x;
-        o3[3 * p + 1] = y;
-        o3[3 * p + 2] = z;
+    float4 a, b;
+    if (ALIGNED) {
+        asm("ld.global.nc.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+            : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)
+            : "l"(g + 2 * (size_t)p));
     } else {
-        o4[p] = make_float4(x, y, z, 0.0f);
+        a = __ldg(g + 2 * (size_t)p);
+        b = __ldg(g + 2 * (size_t)p + 1);
+    }
+    return Guide{a.x, a.y, a.z, a.w, b.x, b.y};
+}
+
+__global__ void __launch_bounds__(256) k_eawt_pack(const float* __restrict__ image, const float* __restrict__ normal,
+                                                   const float* __restrict__ position, float4* __restrict__ c,
+                                                   float4* __restrict__ g, int64_t npx)
+{
+    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < npx; p += (int64_t)gridDim.x * blockDim.x) {
+        const float *i = image + 3 * p, *n = normal + 3 * p, *x = position + 3 * p;
+        c[p] = make_float4(__ldg(i), __ldg(i + 1), __ldg(i + 2), 0.0f);
+        g[2 * p] = make_float4(__ldg(n), __ldg(n + 1), __ldg(n + 2), __ldg(x));
+        g[2 * p + 1] = make_float4(__ldg(x + 1), __ldg(x + 2), 0.0f, 0.0f);
     }
 }
 
-// The level kernels run over a stack of N images of W x H. A thread takes a strip of EAWT_R
-// output pixels of one column spaced `step` rows apart (rows y0 + j step): their 5 x 5 footprints
-// overlap in all but the first and last rows, so the strip reads its (EAWT_R + 4) x 5 taps once
-// each and applies every tap to the outputs it falls on -- (EAWT_R + 4) 5 / EAWT_R tap reads per
-// output instead of 25 (15 for strips of two). Consecutive threads take consecutive columns of the same rows (coalesced
-// tap rows). Each output still sums its taps row by row, column by column.
-// Measured on 20 views of config 3 (forward + adjoint, 3 levels): strips of 2 at 64 registers
-// (4 blocks per SM) 5.29 ms; 4 at 80 (3 blocks, spilling) 5.61; 4 at 128 (2 blocks) 5.59;
-// 2 at 2 blocks 6.18; 8 at 1 block 8.97.
-#ifndef MR_EAWT_R
-#define MR_EAWT_R 2  // outputs per strip
-#endif
+// the adjoint's input at the last level: d_out / k
+__global__ void __launch_bounds__(256) k_eawt_pack_adjoint(const float* __restrict__ d, const float* __restrict__ ik,
+                                                           float4* __restrict__ out, int64_t npx)
+{
+    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < npx; p += (int64_t)gridDim.x * blockDim.x) {
+        const float k = __ldg(ik + p);
+        out[p] = make_float4(__ldg(d + 3 * p) * k, __ldg(d + 3 * p + 1) * k, __ldg(d + 3 * p + 2) * k, 0.0f);
+    }
+}
+
+__device__ __forceinline__ void store3(float* o3, uint32_t p, float x, float y, float z)
+{
+    o3[3 * (size_t)p] = x;
+    o3[3 * (size_t)p + 1] = y;
+    o3[3 * (size_t)p + 2] = z;
+}
+
+// One level over a stack of N images of W x H. A thread takes a strip of two output pixels of one
+// column `step` rows apart: their 5 x 5 footprints overlap in four of six rows, so the strip reads
+// its 6 x 5 taps once each -- 15 tap reads per output instead of 25. A block is 32 columns by 8
+// strips, and strips of one residue of the rows mod `step` follow each other, so that neighbouring
+// warps share tap rows in L1; block and grid are two- and three-dimensional, as the 64-bit
+// divisions of a flat index cost a twelfth of the instructions. The kernel is bound by issue slots
+// (about 28 instructions a tap and output: nine differences, the squared distances, one
+// exponential, the sums) and its code size: the four rows that both outputs use are a loop, not
+// unrolled, as the flat 6 x 5 x 2 body overran the instruction cache (20% of the stalls).
+// 8 images of 800 x 800, three levels, forward / adjoint: 851 / 1097 us with flat strips of two
+// (unrolled, three 16-byte loads a tap and 1 / k read per tap), now 575 / 705.
+// ADJOINT: gout(q) = sum over taps of h w(q, q + tap) gin(q + tap), gin already divided by k, the
+// weights recomputed from the level's recorded input c; the output is divided by the next level's k
+// (ikio). Forward: cout = sum h w c / k, and 1 / k to ikio.
 #ifndef MR_EAWT_MINB
 #define MR_EAWT_MINB 4  // resident 256-thread blocks per SM the register cap aims at
 #endif
-constexpr int EAWT_R = MR_EAWT_R;
+constexpr int EAWT_X = 32, EAWT_Y = 8;
 
-struct Strip {
-    int img, x, y0;
-};
-
-// strip t of the stack: image, column, first row (row block B of EAWT_R step rows, residue ry)
-__device__ __forceinline__ Strip strip_of(int64_t t, int W, int step, int64_t per_img)
+template <bool ADJOINT, bool ALIGNED>
+__global__ void __launch_bounds__(EAWT_X* EAWT_Y, MR_EAWT_MINB)
+    k_eawt_level(const float4* __restrict__ c, const float4* __restrict__ gbuf, const float4* __restrict__ gin, int N,
+                 int W, int H, int lstep, float inv_rt2, float inv_n2, float inv_x2, float4* __restrict__ out,
+                 float* __restrict__ out3, float* __restrict__ ikio)
 {
-    Strip s;
-    s.img = (int)(t / per_img);
-    const int64_t r = t - (int64_t)s.img * per_img;
-    s.x = (int)(r % W);
-    const int64_t sr = r / W;
-    s.y0 = (int)(sr / step) * (EAWT_R * step) + (int)(sr % step);
-    return s;
-}
-
-__device__ __forceinline__ int64_t strips_per_image(int W, int H, int step)
-{
-    return (int64_t)((H + EAWT_R * step - 1) / (EAWT_R * step)) * step * W;
-}
-
-// forward level: cin -> cout (packed, or [N][H][W][3] when out3 is given), and 1 / k
-__global__ void __launch_bounds__(256, MR_EAWT_MINB) k_eawt_level(const float4* __restrict__ cin, const float4* __restrict__ nrm,
-                                                    const float4* __restrict__ pos, int N, int W, int H, int step,
-                                                    float inv_rt2, float inv_n2, float inv_x2, float4* __restrict__ cout,
-                                                    float* __restrict__ out3, float* __restrict__ ikout)
-{
-    const int64_t npx = (int64_t)W * H, per_img = strips_per_image(W, H, step), total = per_img * N;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-        const Strip sp = strip_of(t, W, step, per_img);
-        if (sp.y0 >= H) continue;
-        const int64_t base = (int64_t)sp.img * npx;
-        float4 cp[EAWT_R], np_[EAWT_R], xp[EAWT_R];
-        float ax[EAWT_R], ay[EAWT_R], az[EAWT_R], k[EAWT_R];
+    const int step = 1 << lstep;
+    const uint32_t npx = (uint32_t)W * (uint32_t)H;
+    const int n_strips = ((H + 2 * step - 1) / (2 * step)) * step;
+    const int x = blockIdx.x * EAWT_X + threadIdx.x;
+    if (x >= W) return;
+    const float A = -kLog2e * inv_rt2, B = -kLog2e * inv_n2, C = -kLog2e * inv_x2;
+    for (int img = blockIdx.z; img < N; img += gridDim.z)
+        for (int sr = blockIdx.y * EAWT_Y + threadIdx.y; sr < n_strips; sr += gridDim.y * EAWT_Y) {
+            const int y0 = ((sr >> lstep) << (lstep + 1)) + (sr & (step - 1)), y1 = y0 + step;
+            if (y0 >= H) continue;
+            const uint32_t base = (uint32_t)img * npx;
+            const uint32_t p0 = base + (uint32_t)y0 * (uint32_t)W + (uint32_t)x;
+            const uint32_t p1 = y1 < H ? p0 + (uint32_t)step * (uint32_t)W : p0;
+            const float4 c0 = __ldg(c + p0), c1 = __ldg(c + p1);
+            const Guide g0 = guide_at<ALIGNED>(gbuf, p0), g1 = guide_at<ALIGNED>(gbuf, p1);
+            float3 a0 = f3(0.f, 0.f, 0.f), a1 = a0;
+            float k0 = 0.0f, k1 = 0.0f;
+            auto weight = [&](const float4& cp, const Guide& gp, const float4& cq, const Guide& gq, float lh) {
+                const float dx = cp.x - cq.x, dy = cp.y - cq.y, dz = cp.z - cq.z;
+                const float nx = gp.nx - gq.nx, ny = gp.ny - gq.ny, nz = gp.nz - gq.nz;
+                const float px = gp.x - gq.x, py = gp.y - gq.y, pz = gp.z - gq.z;
+                const float dc = dx * dx + dy * dy + dz * dz, dn = nx * nx + ny * ny + nz * nz,
+                            dp = px * px + py * py + pz * pz;
+                return exp2_approx(fmaf(dc, A, fmaf(dn, B, fmaf(dp, C, lh))));
+            };
+            // the five taps of one row; lh0, lh1: log2 of the row's B3 weight for either output
+            auto row = [&](int qy, bool use0, bool use1, float lh0, float lh1) {
+                if (qy < 0 || qy >= H) return;
 #pragma unroll
-        for (int j = 0; j < EAWT_R; ++j) {
-            const int y = sp.y0 + j * step;
-            const int64_t p = base + (int64_t)min(y, H - 1) * W + sp.x;
-            cp[j] = __ldg(cin + p);
-            np_[j] = __ldg(nrm + p);
-            xp[j] = __ldg(pos + p);
-            ax[j] = ay[j] = az[j] = k[j] = 0.f;
-        }
-#pragma unroll
-        for (int m = 0; m < EAWT_R + 4; ++m) {
-            const int qy = sp.y0 + (m - 2) * step;
-            if (qy < 0 || qy >= H) continue;
-#pragma unroll
-            for (int b = 0; b < 5; ++b) {
-                const int qx = sp.x + (b - 2) * step;
-                if (qx < 0 || qx >= W) continue;
-                const int64_t q = base + (int64_t)qy * W + qx;
-                const float4 cq = __ldg(cin + q), nq = __ldg(nrm + q), xq = __ldg(pos + q);
-#pragma unroll
-                for (int j = 0; j < EAWT_R; ++j) {
-                    const int a = m - j;  // the tap's row in output j's footprint
-                    if (a < 0 || a > 4) continue;
-                    const float e = d2(cp[j], cq) * inv_rt2 + d2(np_[j], nq) * inv_n2 + d2(xp[j], xq) * inv_x2;
-                    const float w = kB3[a] * kB3[b] * __expf(-e);
-                    ax[j] += w * cq.x;
-                    ay[j] += w * cq.y;
-                    az[j] += w * cq.z;
-                    k[j] += w;
+                for (int b = 0; b < 5; ++b) {
+                    const int qx = x + (b - 2) * step;
+                    if (qx < 0 || qx >= W) continue;
+                    const uint32_t q = base + (uint32_t)qy * (uint32_t)W + (uint32_t)qx;
+                    const float4 cq = __ldg(c + q);
+                    const Guide gq = guide_at<ALIGNED>(gbuf, q);
+                    const float4 v = ADJOINT ? __ldg(gin + q) : cq;
+                    if (use0) {
+                        const float w = weight(c0, g0, cq, gq, lh0 + kLogB3[b]);
+                        a0.x += w * v.x;
+                        a0.y += w * v.y;
+                        a0.z += w * v.z;
+                        if (!ADJOINT) k0 += w;
+                    }
+                    if (use1) {
+                        const float w = weight(c1, g1, cq, gq, lh1 + kLogB3[b]);
+                        a1.x += w * v.x;
+                        a1.y += w * v.y;
+                        a1.z += w * v.z;
+                        if (!ADJOINT) k1 += w;
+                    }
                 }
-            }
+            };
+            row(y0 - 2 * step, true, false, kLogB3[0], 0.0f);
+#pragma unroll 1
+            for (int m = 1; m < 5; ++m) row(y0 + (m - 2) * step, true, true, kLogB3[m], kLogB3[m - 1]);
+            if (y1 < H) row(y1 + 2 * step, false, true, 0.0f, kLogB3[4]);
+            auto emit = [&](uint32_t p, const float3& a, float k) {
+                // k >= (6/16)^2: the centre tap has weight 1
+                const float f = ADJOINT ? (ikio ? __ldg(ikio + p) : 1.0f) : 1.0f / k;
+                if (!ADJOINT) ikio[p] = f;
+                if (out3) store3(out3, p, a.x * f, a.y * f, a.z * f);
+                else out[p] = make_float4(a.x * f, a.y * f, a.z * f, 0.0f);
+            };
+            emit(p0, a0, k0);
+            if (y1 < H) emit(p1, a1, k1);
         }
-#pragma unroll
-        for (int j = 0; j < EAWT_R; ++j) {
-            const int y = sp.y0 + j * step;
-            if (y >= H) break;
-            const int64_t p = base + (int64_t)y * W + sp.x;
-            const float ik = 1.0f / k[j];  // k >= (6/16)^2: the centre tap has weight 1
-            store(cout, out3, p, ax[j] * ik, ay[j] * ik, az[j] * ik);
-            ikout[p] = ik;
-        }
-    }
-}
-
-// adjoint level: gout(q) = sum over taps of h w(q, q + tap) gin(q + tap) / k(q + tap), the
-// weights recomputed from the level's recorded input c, 1 / k read from the record
-__global__ void __launch_bounds__(256, MR_EAWT_MINB) k_eawt_level_adjoint(const float4* __restrict__ gin, const float4* __restrict__ c,
-                                                            const float* __restrict__ ikin, const float4* __restrict__ nrm,
-                                                            const float4* __restrict__ pos, int N, int W, int H, int step,
-                                                            float inv_rt2, float inv_n2, float inv_x2,
-                                                            float4* __restrict__ gout, float* __restrict__ out3)
-{
-    const int64_t npx = (int64_t)W * H, per_img = strips_per_image(W, H, step), total = per_img * N;
-    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total; t += (int64_t)gridDim.x * blockDim.x) {
-        const Strip sp = strip_of(t, W, step, per_img);
-        if (sp.y0 >= H) continue;
-        const int64_t base = (int64_t)sp.img * npx;
-        float4 cp[EAWT_R], np_[EAWT_R], xp[EAWT_R];
-        float ax[EAWT_R], ay[EAWT_R], az[EAWT_R];
-#pragma unroll
-        for (int j = 0; j < EAWT_R; ++j) {
-            const int y = sp.y0 + j * step;
-            const int64_t p = base + (int64_t)min(y, H - 1) * W + sp.x;
-            cp[j] = __ldg(c + p);
-            np_[j] = __ldg(nrm + p);
-            xp[j] = __ldg(pos + p);
-            ax[j] = ay[j] = az[j] = 0.f;
-        }
-#pragma unroll
-        for (int m = 0; m < EAWT_R + 4; ++m) {
-            const int qy = sp.y0 + (m - 2) * step;
-            if (qy < 0 || qy >= H) continue;
-#pragma unroll
-            for (int b = 0; b < 5; ++b) {
-                const int qx = sp.x + (b - 2) * step;
-                if (qx < 0 || qx >= W) continue;
-                const int64_t q = base + (int64_t)qy * W + qx;
-                const float4 cq = __ldg(c + q), nq = __ldg(nrm + q), xq = __ldg(pos + q), g = __ldg(gin + q);
-                const float ik = __ldg(ikin + q);
-#pragma unroll
-                for (int j = 0; j < EAWT_R; ++j) {
-                    const int a = m - j;
-                    if (a < 0 || a > 4) continue;
-                    const float e = d2(cp[j], cq) * inv_rt2 + d2(np_[j], nq) * inv_n2 + d2(xp[j], xq) * inv_x2;
-                    const float w = kB3[a] * kB3[b] * __expf(-e) * ik;
-                    ax[j] += w * g.x;
-                    ay[j] += w * g.y;
-                    az[j] += w * g.z;
-                }
-            }
-        }
-#pragma unroll
-        for (int j = 0; j < EAWT_R; ++j) {
-            const int y = sp.y0 + j * step;
-            if (y >= H) break;
-            store(gout, out3, base + (int64_t)y * W + sp.x, ax[j], ay[j], az[j]);
-        }
-    }
 }
 
 // G-buffer: the primary hit through each pixel centre, face normal turned towards the camera
@@ -229,30 +207,42 @@ unsigned grid_for_pixels(int64_t n, int sms)
 
 }  // namespace
 
-void mr_launch_eawt_pack(const float* a, float4* out, int64_t npx, int sms, cudaStream_t st)
+void mr_launch_eawt_pack(const float* image, const float* normal, const float* position, float4* c, float4* g,
+                         int64_t npx, int sms, cudaStream_t st)
 {
-    k_eawt_pack<<<grid_for_pixels(npx, sms), 256, 0, st>>>(a, out, npx);
+    k_eawt_pack<<<grid_for_pixels(npx, sms), 256, 0, st>>>(image, normal, position, c, g, npx);
 }
 
-static int64_t level_strips(int N, int W, int H, int step)
+void mr_launch_eawt_pack_adjoint(const float* d, const float* ik, float4* out, int64_t npx, int sms, cudaStream_t st)
 {
-    return (int64_t)N * ((H + EAWT_R * step - 1) / (EAWT_R * step)) * step * W;
+    k_eawt_pack_adjoint<<<grid_for_pixels(npx, sms), 256, 0, st>>>(d, ik, out, npx);
 }
 
-void mr_launch_eawt_level(const float4* cin, const float4* nrm, const float4* pos, int N, int W, int H, int step,
-                          float inv_rt2, float inv_n2, float inv_x2, float4* cout, float* out3, float* ikout, int sms,
-                          cudaStream_t st)
+template <bool ADJOINT>
+static void launch_level(const float4* c, const float4* g, const float4* gin, int N, int W, int H, int lstep,
+                         float inv_rt2, float inv_n2, float inv_x2, float4* out, float* out3, float* ikio,
+                         cudaStream_t st)
 {
-    k_eawt_level<<<grid_for_pixels(level_strips(N, W, H, step), sms), 256, 0, st>>>(
-        cin, nrm, pos, N, W, H, step, inv_rt2, inv_n2, inv_x2, cout, out3, ikout);
+    const int64_t step = (int64_t)1 << lstep, strips = (H + 2 * step - 1) / (2 * step) * step;
+    const dim3 grid((unsigned)((W + EAWT_X - 1) / EAWT_X),
+                    (unsigned)std::min<int64_t>((strips + EAWT_Y - 1) / EAWT_Y, 65535),
+                    (unsigned)std::min(N, 65535));
+    const bool aligned = (reinterpret_cast<uintptr_t>(g) & 31) == 0;
+    (aligned ? k_eawt_level<ADJOINT, true> : k_eawt_level<ADJOINT, false>)<<<grid, dim3(EAWT_X, EAWT_Y), 0, st>>>(
+        c, g, gin, N, W, H, lstep, inv_rt2, inv_n2, inv_x2, out, out3, ikio);
 }
 
-void mr_launch_eawt_level_adjoint(const float4* gin, const float4* c, const float* ikin, const float4* nrm,
-                                  const float4* pos, int N, int W, int H, int step, float inv_rt2, float inv_n2,
-                                  float inv_x2, float4* gout, float* out3, int sms, cudaStream_t st)
+void mr_launch_eawt_level(const float4* c, const float4* g, int N, int W, int H, int lstep, float inv_rt2, float inv_n2,
+                          float inv_x2, float4* cout, float* out3, float* ikout, cudaStream_t st)
 {
-    k_eawt_level_adjoint<<<grid_for_pixels(level_strips(N, W, H, step), sms), 256, 0, st>>>(
-        gin, c, ikin, nrm, pos, N, W, H, step, inv_rt2, inv_n2, inv_x2, gout, out3);
+    launch_level<false>(c, g, nullptr, N, W, H, lstep, inv_rt2, inv_n2, inv_x2, cout, out3, ikout, st);
+}
+
+void mr_launch_eawt_level_adjoint(const float4* gin, const float4* c, const float4* g, int N, int W, int H, int lstep,
+                                  float inv_rt2, float inv_n2, float inv_x2, float4* gout, float* out3,
+                                  const float* ik_next, cudaStream_t st)
+{
+    launch_level<true>(c, g, gin, N, W, H, lstep, inv_rt2, inv_n2, inv_x2, gout, out3, const_cast<float*>(ik_next), st);
 }
 
 void mr_launch_gbuffer(const SceneDev& s, const ViewDev& v, float* nrm, float* pos, int sms, cudaStream_t st)

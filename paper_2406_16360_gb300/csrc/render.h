@@ -104,13 +104,16 @@ void mr_launch_trace_rays(const SceneDev& s, const float* rays, const int32_t* s
                           int32_t* hit_tri, float* hit_tuv, int sms, cudaStream_t st);
 
 // denoise.cu: EAWT levels, their adjoints, the pixel-centre G-buffer
-void mr_launch_eawt_pack(const float* a, float4* out, int64_t npx, int sms, cudaStream_t st);
-void mr_launch_eawt_level(const float4* cin, const float4* nrm, const float4* pos, int N, int W, int H, int step,
-                          float inv_rt2, float inv_n2, float inv_x2, float4* cout, float* out3, float* ikout, int sms,
-                          cudaStream_t st);
-void mr_launch_eawt_level_adjoint(const float4* gin, const float4* c, const float* ikin, const float4* nrm,
-                                  const float4* pos, int N, int W, int H, int step, float inv_rt2, float inv_n2,
-                                  float inv_x2, float4* gout, float* out3, int sms, cudaStream_t st);
+void mr_launch_eawt_pack(const float* image, const float* normal, const float* position, float4* c, float4* g,
+                         int64_t npx, int sms, cudaStream_t st);
+void mr_launch_eawt_pack_adjoint(const float* d, const float* ik, float4* out, int64_t npx, int sms, cudaStream_t st);
+// level lstep (taps 2^lstep pixels apart); g: 32-byte G-buffer records
+void mr_launch_eawt_level(const float4* c, const float4* g, int N, int W, int H, int lstep, float inv_rt2, float inv_n2,
+                          float inv_x2, float4* cout, float* out3, float* ikout, cudaStream_t st);
+// gin: the gradient over the level's k; ik_next: 1 / k of the level below, null at the first
+void mr_launch_eawt_level_adjoint(const float4* gin, const float4* c, const float4* g, int N, int W, int H, int lstep,
+                                  float inv_rt2, float inv_n2, float inv_x2, float4* gout, float* out3,
+                                  const float* ik_next, cudaStream_t st);
 void mr_launch_gbuffer(const SceneDev& s, const ViewDev& v, float* nrm, float* pos, int sms, cudaStream_t st);
 // regular.cu: mesh regularisers over the scene's edge list (built by mr_edges_build)
 void mr_launch_material_smoothness(const SceneDev& s, const ViewDev& v, uint32_t view_index, const Rng& rng,
