@@ -18,7 +18,7 @@
 #define MR_SHADE_MINB 4
 #endif
 #ifndef MR_BWD_MINB
-#define MR_BWD_MINB 4
+#define MR_BWD_MINB 2
 #endif
 #ifndef MR_TRACE_MINB
 #define MR_TRACE_MINB 0  // the batched closest-hit and shadow-ray kernels (0: no minimum)
@@ -93,6 +93,7 @@ struct SceneDev {
     const float* albedo;      // [th][tw][3]
     const float* rough;       // [th][tw]
     const float* metal;       // [th][tw]
+    const float4* tex8;       // [th][tw][2] (albedo, roughness) (metallic, -) of this call, null where not packed
     const float4* env_texel;  // [eh][ew]: (r, g, b, prob * ew * eh)
     const float4* env_row;    // [eh]: (cos th_r, sin th_r, 2 pi^2 total / (ew eh sin th_r), 0) at row centres
     const float2* env_col;    // [ew]: (cos psi_c, sin psi_c), psi = 2 pi u - pi at column centres
@@ -1050,9 +1051,27 @@ struct Shade {
     float nsg;
 };
 
+// albedo, roughness and metallic of one texel; PACKED: from the 32-byte records of s.tex8
+template <bool PACKED>
+__device__ __forceinline__ void texel_at(const SceneDev& s, int i, float (&x)[5])
+{
+    if (PACKED) {
+        float pad[3];
+        asm("ld.global.nc.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+            : "=f"(x[0]), "=f"(x[1]), "=f"(x[2]), "=f"(x[3]), "=f"(x[4]), "=f"(pad[0]), "=f"(pad[1]), "=f"(pad[2])
+            : "l"(s.tex8 + 2 * (size_t)i));
+    } else {
+        x[0] = __ldg(s.albedo + 3 * (size_t)i);
+        x[1] = __ldg(s.albedo + 3 * (size_t)i + 1);
+        x[2] = __ldg(s.albedo + 3 * (size_t)i + 2);
+        x[3] = __ldg(s.rough + i);
+        x[4] = __ldg(s.metal + i);
+    }
+}
+
 // INTERP = false compiles the interpolated-normal path out (kernels launched for scenes that
 // all use face normals); INTERP = true follows the scene (s.vnrm)
-template <bool INTERP = true>
+template <bool INTERP = true, bool PACKED = false>
 __device__ __forceinline__ void shade_at(const SceneDev& s, int tri, float u, float v, float3 d, Shade& sh)
 {
     float3 v0;
@@ -1090,13 +1109,14 @@ __device__ __forceinline__ void shade_at(const SceneDev& s, int tri, float u, fl
     float r = 0.0f, m = 0.0f;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        const int i = sh.tp.idx[k];
         const float w = sh.tp.w[k];
-        a.x += w * __ldg(s.albedo + 3 * (size_t)i);
-        a.y += w * __ldg(s.albedo + 3 * (size_t)i + 1);
-        a.z += w * __ldg(s.albedo + 3 * (size_t)i + 2);
-        r += w * __ldg(s.rough + i);
-        m += w * __ldg(s.metal + i);
+        float x[5];
+        texel_at<PACKED>(s, sh.tp.idx[k], x);
+        a.x += w * x[0];
+        a.y += w * x[1];
+        a.z += w * x[2];
+        r += w * x[3];
+        m += w * x[4];
     }
     sh.m.alb = a;
     sh.m.rough = r;

@@ -423,27 +423,31 @@ __global__ void __launch_bounds__(256) k_resolve_all(const ViewDev* __restrict__
 // adjoint (PRIMARY mode): replay of the primary vertex from the tape and the random stream
 // ---------------------------------------------------------------------------------------
 // reverse-mode derivative of Q = f_r(wo, wi) max(0, n.wi) (per channel) for the upstream
-// gradient gq: gm = (d/d albedo[3], d/d roughness, d/d metallic, d/d n[3]). DEMOD: of the
-// demodulated lobes (diffuse reflectance 1: no albedo or metallic term through it)
+// gradient gq: gm += (d/d albedo[3], d/d roughness, d/d metallic, d/d n[3]); returns Q. DEMOD: of
+// the demodulated lobes (diffuse reflectance 1: no albedo or metallic term through it)
 template <bool DEMOD = false>
-__device__ __forceinline__ void brdf_cos_adjoint(float3 n, float3 wo, float3 wi, const Material& m, float3 gq,
-                                                 float gm[8])
+__device__ __forceinline__ float3 brdf_cos_adjoint(float3 n, float3 wo, float3 wi, const Material& m, float3 gq,
+                                                   float gm[8])
 {
+    float3 Q = f3(0.f, 0.f, 0.f);
     const float co = dot(n, wo), ci = dot(n, wi);
-    if (co <= 0.0f || ci <= 0.0f) return;
+    if (co <= 0.0f || ci <= 0.0f) return Q;
     const float r = m.rough;
     const float a = alpha_of(r), a2 = a * a;
     const float3 h = normalize(add(wo, wi));
     const float cnh = dot(n, h), coh = dot(wo, h);
     const float k = ggx_k(n, h, cnh, a2);  // d k / d cnh = 2 cnh (a^2 - 1)
-    const float D = a2 / (MR_PI * k * k);
+    const float rk2 = 1.0f / (MR_PI * k * k), rk3 = rk2 / k;
+    const float D = a2 * rk2;
     const float Ao = smith_a(a2, co), Ai = smith_a(a2, ci);
-    const float den = ci * Ao + co * Ai;
-    const float vis = 0.5f / den;
+    const float rAo = 1.0f / Ao, rAi = 1.0f / Ai;
+    const float den = ci * Ao + co * Ai, rden = 1.0f / den;
+    const float vis = 0.5f * rden;
     const float om = 1.0f - coh;
     const float w5 = (om * om) * (om * om) * om;
     const float alb[3] = {m.alb.x, m.alb.y, m.alb.z};
     const float g[3] = {gq.x, gq.y, gq.z};
+    float q[3];
     float S = 0.0f, g_ci = 0.0f, g_m = 0.0f;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -455,22 +459,25 @@ __device__ __forceinline__ void brdf_cos_adjoint(float3 n, float3 wo, float3 wi,
         gm[c] += gkd * (1.0f - m.metal) + gF * (1.0f - w5) * m.metal;
         g_m += -gkd * alb[c] + gF * (1.0f - w5) * (alb[c] - 0.04f);
         S += g[c] * F;
-        g_ci += g[c] * (kd * MR_INV_PI + D * vis * F);  // the trailing cosine
+        const float f = kd * MR_INV_PI + D * vis * F;
+        q[c] = f * ci;
+        g_ci += g[c] * f;  // the trailing cosine
     }
+    Q = f3(q[0], q[1], q[2]);
     const float gDV = S * ci;
     const float gD = gDV * vis, gvis = gDV * D;
-    const float gden = gvis * (-0.5f / (den * den));
-    const float k3 = MR_PI * k * k * k;
-    float g_a = gD * (2.0f * a / (MR_PI * k * k) - 4.0f * a * a2 * cnh * cnh / k3);
-    const float g_cnh = gD * (-4.0f * a2 * cnh * (a2 - 1.0f) / k3);
-    g_ci += gden * (Ao + co * (1.0f - a2) * ci / Ai);
-    const float g_co = gden * (Ai + ci * (1.0f - a2) * co / Ao);
-    g_a += gden * (ci * a * (1.0f - co * co) / Ao + co * a * (1.0f - ci * ci) / Ai);
+    const float gden = -gvis * vis * rden;
+    float g_a = gD * (2.0f * a * rk2 - 4.0f * a * a2 * cnh * cnh * rk3);
+    const float g_cnh = gD * (-4.0f * a2 * cnh * (a2 - 1.0f) * rk3);
+    g_ci += gden * (Ao + co * (1.0f - a2) * ci * rAi);
+    const float g_co = gden * (Ai + ci * (1.0f - a2) * co * rAo);
+    g_a += gden * (ci * a * (1.0f - co * co) * rAo + co * a * (1.0f - ci * ci) * rAi);
     gm[3] += (r * r > 1e-3f) ? g_a * 2.0f * r : 0.0f;
     gm[4] += g_m;
     gm[5] += g_ci * wi.x + g_co * wo.x + g_cnh * h.x;
     gm[6] += g_ci * wi.y + g_co * wo.y + g_cnh * h.y;
     gm[7] += g_ci * wi.z + g_co * wo.z + g_cnh * h.z;
+    return Q;
 }
 
 struct EmitEnv {
@@ -509,6 +516,12 @@ struct EmitVert {
     }
 };
 
+// the same into the packed accumulators (GradDev::ptex, penv, pvert): one 16-byte reduction where
+// three to five 4-byte ones would go
+__device__ __forceinline__ void red4(float4* p, float a, float b, float c, float d)
+{
+    asm volatile("red.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
+}
 // The FULL-mode vertex loops call the heavy helpers (shading point, BRDF, its adjoint, the
 // candidate redraw, the gradient scatters) through these wrappers; MR_FULL_NOINLINE=1 makes
 // them single out-of-line copies. That helped while one kernel held the primary and the later
@@ -518,9 +531,6 @@ struct EmitVert {
 #endif
 #ifndef MR_FULL_MINB
 #define MR_FULL_MINB 2  // resident blocks of 256 threads per SM for the FULL-mode adjoint
-#endif
-#ifndef MR_FULL_SPLIT
-#define MR_FULL_SPLIT 1  // later vertices in their own kernel over samples grouped by vertex count
 #endif
 #define MR_FULL_CHUNK (1u << 25)  // samples classified per pass
 #if MR_FULL_NOINLINE
@@ -536,9 +546,9 @@ MR_FULL_FN void fv_shade(const SceneDev& s, int tri, float u, float v, float3 d,
 
 MR_FULL_FN float3 fv_brdf(float3 n, float3 wo, float3 wi, const Material& m) { return brdf_cos(n, wo, wi, m); }
 
-MR_FULL_FN void fv_brdf_adjoint(float3 n, float3 wo, float3 wi, const Material& m, float3 gq, float* gm)
+MR_FULL_FN float3 fv_brdf_adjoint(float3 n, float3 wo, float3 wi, const Material& m, float3 gq, float* gm)
 {
-    brdf_cos_adjoint(n, wo, wi, m, gq, gm);
+    return brdf_cos_adjoint(n, wo, wi, m, gq, gm);
 }
 
 // the selected candidate of vertex b, redrawn from its Philox block
@@ -656,14 +666,13 @@ __device__ __forceinline__ void full_backward(const SceneDev& s, const Rng& rng,
                 float3 y;
                 int ytex;
                 fv_candidate(s, rng, pixel, smp, view, (uint32_t)b, (uint32_t)cand, y, ytex);
-                const float3 fy = fv_brdf(sh.n, wo, y, sh.m);
                 const float4 L = __ldg(s.env_texel + ytex);
+                const float3 gf = f3(gI.x * bt.x * wv, gI.y * bt.y * wv, gI.z * bt.z * wv);
+                const float3 fy = fv_brdf_adjoint(sh.n, wo, y, sh.m, hmul(gf, xyz(L)), gm);
                 env_key = ytex;
-                env_v[0] = gI.x * bt.x * wv * fy.x;
-                env_v[1] = gI.y * bt.y * wv * fy.y;
-                env_v[2] = gI.z * bt.z * wv * fy.z;
-                fv_brdf_adjoint(sh.n, wo, y, sh.m, f3(gI.x * bt.x * wv * L.x, gI.y * bt.y * wv * L.y, gI.z * bt.z * wv * L.z),
-                                gm);
+                env_v[0] = gf.x * fy.x;
+                env_v[1] = gf.y * fy.y;
+                env_v[2] = gf.z * fy.z;
             }
             const float p = __uint_as_float(*vx_at(tp, b, VX_P, g));
             if (p > 0.0f && (lin.x != 0.0f || lin.y != 0.0f || lin.z != 0.0f)) {
@@ -689,20 +698,24 @@ __device__ __forceinline__ void full_backward(const SceneDev& s, const Rng& rng,
     }
 }
 
-// Adjoint of every sample. PRIMARY mode (FULL = false): the primary vertex, replayed from the
-// tape. FULL mode: in addition the vertices b >= 1 from their tape records (see
-// full_vertices below). DEMOD (PRIMARY only): of the demodulated lighting of the monochrome
-// light regulariser instead of the radiance -- the same primary-vertex terms with the
-// demodulated lobes, and nothing for an escaping primary ray. All 32 lanes of a warp run the
-// same number of rounds, so the warp-collective scatters see every lane.
-template <bool FULL, int MINB, bool INTERP, bool DEMOD = false>
-__global__ void __launch_bounds__(256, MINB) k_backward(const SceneDev* __restrict__ scenes,
-                                                        const ViewDev* __restrict__ views, int n_views, uint64_t total,
-                                                        Rng rng, const float* const* __restrict__ d_images,
-                                                        const GradDev* __restrict__ grads, const void* tape, int nvx,
-                                                        unsigned long long* counters)
+// PRIMARY-mode adjoint of every sample: the primary vertex, replayed from the tape. DEMOD: of the
+// demodulated lighting of the monochrome light regulariser instead of the radiance -- the same
+// primary-vertex terms with the demodulated lobes, and nothing for an escaping primary ray. PACKED:
+// materials read from SceneDev::tex8 (one 32-byte load a tap instead of five 4-byte ones) and
+// gradients reduced into GradDev's packed accumulators, which k_grads_unpack adds to the caller's
+// arrays; 32-bit sums as before. Bound by the latency of the tape's and the gathers' loads, which is
+// why the tape's words are all read first and two blocks of 128 registers an SM beat four of 64
+// (9.1 against 10.8 ms on 12 views of config 3, 123 M samples; 14.6 ms with five loads a tap,
+// 4-byte atomics, the words read where they are used and four blocks). All 32 lanes of a warp run the same number of rounds, so the
+// warp-collective scatters see every lane.
+template <bool INTERP, bool DEMOD, bool PACKED>
+__global__ void __launch_bounds__(256, MR_BWD_MINB) k_backward(const SceneDev* __restrict__ scenes,
+                                                               const ViewDev* __restrict__ views, int n_views,
+                                                               uint64_t total, Rng rng,
+                                                               const float* const* __restrict__ d_images,
+                                                               const GradDev* __restrict__ grads, const void* tape,
+                                                               int nvx, unsigned long long* counters)
 {
-    static_assert(!(FULL && DEMOD), "the demodulated lighting is differentiated in PRIMARY mode only");
     const TapeDev tp = tape_of(const_cast<void*>(tape), total, nvx);
     const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
     const uint64_t rounds = (total + stride - 1) / stride;
@@ -710,23 +723,18 @@ __global__ void __launch_bounds__(256, MINB) k_backward(const SceneDev* __restri
     for (uint64_t r = 0; r < rounds; ++r) {
         const uint64_t g = r * stride + blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
         const bool live = g < total;
-        int env_key = -1, tex_key[4] = {-1, -1, -1, -1}, vert_key[3] = {-1, -1, -1};
+        int env_key = -1, tex_key[4] = {-1, -1, -1, -1}, vert_key[3] = {-1, -1, -1}, tri_key = -1;
         float env_v[3] = {0.f, 0.f, 0.f};
         float tex_v[4][5];
         float vert_v[3][3];
         float3 gS = f3(0.f, 0.f, 0.f);  // d loss / d S of the interpolated normal
         float bw_u = 0.0f, bw_v = 0.0f;
         int scene_id = 0;
-        // FULL mode: the later vertices' throughput, direct light and continuation factor
-        int nv = 0;
-        float3 gI_f = f3(0.f, 0.f, 0.f);
-        float3 vbeta[FULL ? MR_FULL_MAXV : 1], vdir[FULL ? MR_FULL_MAXV : 1], vfcp[FULL ? MR_FULL_MAXV : 1];
-        uint32_t f_pixel = 0, f_smp = 0, f_view = 0;
         if (live) {
             int vi;
             const ViewDev& v = view_of(views, n_views, g, vi);
             scene_id = v.scene;
-            const SceneDev s = scenes[v.scene];
+            const SceneDev& s = scenes[v.scene];
             const uint32_t sid = (uint32_t)(g - v.offset);
             const uint32_t pixel = sid / (uint32_t)v.spp, smp = sid % (uint32_t)v.spp;
             const float* dimg = d_images[vi];
@@ -737,9 +745,16 @@ __global__ void __launch_bounds__(256, MINB) k_backward(const SceneDev* __restri
                 ++n_diff;
                 const int px = (int)(pixel % (uint32_t)v.width), py = (int)(pixel / (uint32_t)v.width);
                 const uint4 xc = rng.draw(pixel, smp, (uint32_t)v.index, 0u, PURPOSE_CAMERA, 0u);
+                const int tri = tp.tri[g];
+                // the directions the forward drew: the selected candidate's (with its texel and V W)
+                // and the continuation's (L_ind != 0 implies it was taken); meaningless, and not
+                // used, where the sample has none
+                const int cand = tp.cand[g], ytex = tp.ytex[g];
+                const float wv = tp.wv[g], pind = tp.pind[g];
+                const float3 li = f3(tp.lind[0][g], tp.lind[1][g], tp.lind[2][g]);
+                const float3 y = f3(tp.y[0][g], tp.y[1][g], tp.y[2][g]), wc = f3(tp.wc[0][g], tp.wc[1][g], tp.wc[2][g]);
                 const float3 o = f3(v.c2w[3], v.c2w[7], v.c2w[11]);
                 const float3 d = camera_dir(v, px, py, u24(xc.x), u24(xc.y));
-                const int tri = tp.tri[g];
                 if (tri < 0) {
                     if (!DEMOD) {
                         env_key = env_texel_of(s, d);
@@ -748,49 +763,38 @@ __global__ void __launch_bounds__(256, MINB) k_backward(const SceneDev* __restri
                         env_v[2] = gI.z;
                     }
                 } else {
+                    tri_key = tri;
                     float3 v0, e1, e2;
                     int tchk;
                     load_tri(s, __ldg(s.leaf_of + tri), v0, e1, e2, tchk);
                     float t, u, vv;
                     tri_solve(o, d, v0, e1, e2, t, u, vv);
                     Shade sh;
-                    shade_at<INTERP>(s, tri, u, vv, d, sh);
+                    shade_at<INTERP, PACKED>(s, tri, u, vv, d, sh);
                     const float3 wo = f3(-d.x, -d.y, -d.z);
                     float gm[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-                    const int cand = tp.cand[g];
-                    const float wv = tp.wv[g];
-                    if (cand >= 0 && wv != 0.0f) {
-                        // the selected candidate's direction and texel, as the forward drew them
-                        const float3 y = f3(tp.y[0][g], tp.y[1][g], tp.y[2][g]);
-                        const int ytex = tp.ytex[g];
-                        const float3 fc = brdf_cos<DEMOD>(sh.n, wo, y, sh.m);
-                        const float4 L = __ldg(s.env_texel + ytex);
-                        env_key = ytex;
-                        env_v[0] = gI.x * wv * fc.x;
-                        env_v[1] = gI.y * wv * fc.y;
-                        env_v[2] = gI.z * wv * fc.z;
-                        brdf_cos_adjoint<DEMOD>(sh.n, wo, y, sh.m, f3(gI.x * wv * L.x, gI.y * wv * L.y, gI.z * wv * L.z),
-                                                gm);
-                    }
-                    const float3 li = f3(tp.lind[0][g], tp.lind[1][g], tp.lind[2][g]);
-                    if (v.bounces > 1 && (li.x != 0.0f || li.y != 0.0f || li.z != 0.0f)) {
-                        // the continuation the forward drew (L_ind != 0 implies it was taken)
-                        const float3 wc = f3(tp.wc[0][g], tp.wc[1][g], tp.wc[2][g]);
-                        const float pind = tp.pind[g];
-                        if (FULL && pind > 0.0f) {
-                            // throughput into vertex 1, then the later vertices' forward pass
-                            const float3 fc0 = brdf_cos(sh.n, wo, wc, sh.m);
-                            gI_f = gI;
-                            f_pixel = pixel;
-                            f_smp = smp;
-                            f_view = (uint32_t)v.index;
-                            nv = full_forward(s, rng, tp, g, pixel, smp, (uint32_t)v.index, v.bounces,
-                                              f3(fc0.x / pind, fc0.y / pind, fc0.z / pind), wc, vbeta, vdir, vfcp);
+                    // (one loop body for both directions keeps the kernel inside the instruction cache)
+#pragma unroll 1
+                    for (int k = 0; k < 2; ++k) {
+                        float3 wi = wc, L = li;
+                        float f;
+                        if (k == 0) {
+                            if (cand < 0 || wv == 0.0f) continue;
+                            wi = y;
+                            env_key = ytex;
+                            L = xyz(__ldg(s.env_texel + ytex));
+                            f = wv;
+                        } else {
+                            if (v.bounces <= 1 || (li.x == 0.0f && li.y == 0.0f && li.z == 0.0f) || !(pind > 0.0f)) continue;
+                            f = 1.0f / pind;
                         }
-                        if (pind > 0.0f)
-                            brdf_cos_adjoint<DEMOD>(sh.n, wo, wc, sh.m,
-                                                    f3(gI.x * li.x / pind, gI.y * li.y / pind, gI.z * li.z / pind),
-                                                    gm);
+                        const float3 gf = mul(gI, f);
+                        const float3 Q = brdf_cos_adjoint<DEMOD>(sh.n, wo, wi, sh.m, hmul(gf, L), gm);
+                        if (k == 0) {
+                            env_v[0] = gf.x * Q.x;
+                            env_v[1] = gf.y * Q.y;
+                            env_v[2] = gf.z * Q.z;
+                        }
                     }
                     // textures (bilinear) and the texture coordinate
                     const Taps& tpz = sh.tp;
@@ -802,9 +806,9 @@ __global__ void __launch_bounds__(256, MINB) k_backward(const SceneDev* __restri
                         tex_key[q] = ti;
 #pragma unroll
                         for (int c = 0; c < 5; ++c) tex_v[q][c] = w * gm[c];
-                        dt[q] = gm[0] * __ldg(s.albedo + 3 * (size_t)ti) + gm[1] * __ldg(s.albedo + 3 * (size_t)ti + 1) +
-                                gm[2] * __ldg(s.albedo + 3 * (size_t)ti + 2) + gm[3] * __ldg(s.rough + ti) +
-                                gm[4] * __ldg(s.metal + ti);
+                        float x[5];
+                        texel_at<PACKED>(s, ti, x);
+                        dt[q] = gm[0] * x[0] + gm[1] * x[1] + gm[2] * x[2] + gm[3] * x[3] + gm[4] * x[4];
                     }
                     // derivative of the bilinear lookup along the texture coordinate, as texel
                     // differences (exactly zero across clamped or equal texels)
@@ -842,10 +846,10 @@ __global__ void __launch_bounds__(256, MINB) k_backward(const SceneDev* __restri
                     for (int c = 0; c < 3; ++c) gvx[c] = mul(z, -bw[c]);
                     if (!sh.interp) {
                         // n = sign * N / |N|, N = e1 x e2
-                        const float Nl = sqrtf(dot(sh.N, sh.N));
-                        const float3 Nh = mul(sh.N, 1.0f / Nl);
+                        const float rN = 1.0f / sqrtf(dot(sh.N, sh.N));
+                        const float3 Nh = mul(sh.N, rN);
                         const float3 gNh = mul(f3(gm[5], gm[6], gm[7]), sh.sign);
-                        const float3 gN = mul(sub(gNh, mul(Nh, dot(Nh, gNh))), 1.0f / Nl);
+                        const float3 gN = mul(sub(gNh, mul(Nh, dot(Nh, gNh))), rN);
                         const float3 ge1 = cross(e2, gN), ge2 = cross(gN, e1);
                         gvx[0] = sub(gvx[0], add(ge1, ge2));
                         gvx[1] = add(gvx[1], ge1);
@@ -861,51 +865,106 @@ __global__ void __launch_bounds__(256, MINB) k_backward(const SceneDev* __restri
                 }
             }
         }
-        // scatters are keyed per scene; lanes of other scenes never share a key group
-        // because the key is combined with the scene id in the match
-        const GradDev gd = grads[scene_id];
-        float* const gvn = (INTERP && gd.verts) ? scenes[scene_id].gvn : nullptr;  // interpolated normals only
-        const unsigned same_scene = __match_any_sync(MR_FULL, scene_id);
-        if (same_scene == MR_FULL) {
-            scatter_agg<3>(env_key, env_v, EmitEnv{gd.env});
+        // one scene's lanes at a time (a warp rarely holds two), so that keys are that scene's
+        for (unsigned todo = MR_FULL; todo;) {
+            const int sid = __shfl_sync(MR_FULL, scene_id, __ffs(todo) - 1);
+            const bool mine = scene_id == sid;
+            todo &= ~__ballot_sync(MR_FULL, mine);
+            const GradDev& gd = grads[sid];
+            if (PACKED) {
+                // (candidates of a warp rarely share a texel: aggregating them costs more than it saves)
+                if (mine && env_key >= 0) red4(gd.penv + env_key, env_v[0], env_v[1], env_v[2], 0.0f);
+                // taps by footprint (its first texel and whether it is clamped in x and y), corners by
+                // triangle: one match and one chain of shuffles for all their sums
+                const int foot = (mine && tex_key[0] >= 0) ? (tex_key[0] << 2) + (tex_key[1] != tex_key[0]) +
+                                                                 2 * (tex_key[2] != tex_key[0])
+                                                           : -1;
+                float tv[20], cv[9];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) scatter_agg<5>(tex_key[q], tex_v[q], EmitTex{gd.albedo, gd.rough, gd.metal});
+                for (int q = 0; q < 20; ++q) tv[q] = tex_v[q / 5][q % 5];
 #pragma unroll
-            for (int c = 0; c < 3; ++c) scatter_agg<3>(vert_key[c], vert_v[c], EmitVert{gd.verts});
+                for (int q = 0; q < 9; ++q) cv[q] = vert_v[q / 3][q % 3];
+                scatter_agg<20>(foot, tv, [&](int, const float (&x)[20]) {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        float4* const t = gd.ptex + 2 * (size_t)tex_key[q];
+                        red4(t, x[5 * q], x[5 * q + 1], x[5 * q + 2], x[5 * q + 3]);
+                        atomicAdd(&t[1].x, x[5 * q + 4]);
+                    }
+                });
+                scatter_agg<9>(mine ? tri_key : -1, cv, [&](int, const float (&x)[9]) {
+#pragma unroll
+                    for (int c = 0; c < 3; ++c)
+                        if (vert_key[c] >= 0) red4(gd.pvert + vert_key[c], x[3 * c], x[3 * c + 1], x[3 * c + 2], 0.0f);
+                });
+            } else {
+                scatter_agg<3>(mine ? env_key : -1, env_v, EmitEnv{gd.env});
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    scatter_agg<5>(mine ? tex_key[q] : -1, tex_v[q], EmitTex{gd.albedo, gd.rough, gd.metal});
+#pragma unroll
+                for (int c = 0; c < 3; ++c) scatter_agg<3>(mine ? vert_key[c] : -1, vert_v[c], EmitVert{gd.verts});
+            }
+            float* const gvn = (INTERP && gd.verts) ? scenes[sid].gvn : nullptr;  // interpolated normals only
             if (gvn) {
                 const float bw[3] = {1.0f - bw_u - bw_v, bw_u, bw_v};
 #pragma unroll
                 for (int c = 0; c < 3; ++c) {
                     const float gv3[3] = {gS.x * bw[c], gS.y * bw[c], gS.z * bw[c]};
-                    scatter_agg<3>(vert_key[c], gv3, EmitVert{gvn});
+                    scatter_agg<3>(mine ? vert_key[c] : -1, gv3, EmitVert{gvn});
                 }
             }
-        } else {
-            if (env_key >= 0) EmitEnv{gd.env}(env_key, env_v);
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-                if (tex_key[q] >= 0) EmitTex{gd.albedo, gd.rough, gd.metal}(tex_key[q], tex_v[q]);
-#pragma unroll
-            for (int c = 0; c < 3; ++c)
-                if (vert_key[c] >= 0) EmitVert{gd.verts}(vert_key[c], vert_v[c]);
-            if (gvn) {
-                const float bw[3] = {1.0f - bw_u - bw_v, bw_u, bw_v};
-#pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    const float gv3[3] = {gS.x * bw[c], gS.y * bw[c], gS.z * bw[c]};
-                    if (vert_key[c] >= 0) EmitVert{gvn}(vert_key[c], gv3);
-                }
-            }
-        }
-        if (FULL) {
-            const SceneDev* sp = scenes + scene_id;
-            full_backward(*sp, rng, tp, g, f_pixel, f_smp, f_view, nv, gI_f, vbeta, vdir, vfcp, gd,
-                          same_scene == MR_FULL);
         }
     }
     if (DEMOD) return;  // counters[4] counts the samples of mirres_backward
     for (int off = 16; off > 0; off >>= 1) n_diff += __shfl_xor_sync(MR_FULL, n_diff, off);
     if (lane_id() == 0 && n_diff) atomicAdd(counters + 4, n_diff);
+}
+
+// albedo, roughness and metallic side by side: one 32-byte record per texel
+__global__ void __launch_bounds__(256) k_tex_pack(const SceneDev* __restrict__ scenes)
+{
+    const SceneDev& s = scenes[blockIdx.y];
+    const float *albedo = s.albedo, *rough = s.rough, *metal = s.metal;
+    float4* const out = const_cast<float4*>(s.tex8);
+    const uint32_t n = (uint32_t)s.tw * (uint32_t)s.th;
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const float* a = albedo + 3 * (size_t)i;
+        out[2 * (size_t)i] = make_float4(__ldg(a), __ldg(a + 1), __ldg(a + 2), __ldg(rough + i));
+        out[2 * (size_t)i + 1] = make_float4(__ldg(metal + i), 0.f, 0.f, 0.f);
+    }
+}
+
+// every scene's packed accumulators added to the caller's gradient arrays
+__global__ void __launch_bounds__(256) k_grads_unpack(const SceneDev* __restrict__ scenes, const GradDev* __restrict__ grads)
+{
+    const SceneDev& s = scenes[blockIdx.y];
+    const GradDev g = grads[blockIdx.y];
+    const uint32_t n_tex = (uint32_t)s.tw * (uint32_t)s.th, n_env = (uint32_t)s.ew * (uint32_t)s.eh, n_verts = (uint32_t)s.n_verts;
+    const uint64_t n = (uint64_t)n_tex + n_env + n_verts;
+    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
+        float* dst;
+        float4 v;
+        if (i < n_tex) {
+            v = __ldcs(g.ptex + 2 * i);
+            if (g.rough) g.rough[i] += v.w;
+            if (g.metal) g.metal[i] += __ldcs(g.ptex + 2 * i + 1).x;
+            dst = g.albedo ? g.albedo + 3 * i : nullptr;
+        } else if (i < (uint64_t)n_tex + n_env) {
+            const uint64_t k = i - n_tex;
+            v = __ldcs(g.penv + k);
+            dst = g.env ? g.env + 3 * k : nullptr;
+        } else {
+            const uint64_t k = i - n_tex - n_env;
+            v = __ldcs(g.pvert + k);
+            dst = g.verts ? g.verts + 3 * k : nullptr;
+        }
+        if (dst) {
+            dst[0] += v.x;
+            dst[1] += v.y;
+            dst[2] += v.z;
+        }
+    }
 }
 
 // ---------------------------------------------------------------------------------------
@@ -953,7 +1012,8 @@ __device__ __forceinline__ float3 light_sample(const SceneDev& s, const ViewDev&
     const float pind = tp.pind[g];
     if (v.bounces > 1 && (li.x != 0.0f || li.y != 0.0f || li.z != 0.0f) && pind > 0.0f) {
         const float3 fc = brdf_cos<true>(sh.n, wo, f3(tp.wc[0][g], tp.wc[1][g], tp.wc[2][g]), sh.m);
-        acc = add(acc, f3(fc.x / pind * li.x, fc.y / pind * li.y, fc.z / pind * li.z));
+        const float rp = 1.0f / pind;
+        acc = add(acc, f3(fc.x * rp * li.x, fc.y * rp * li.y, fc.z * rp * li.z));
     }
     return acc;
 }
@@ -1363,18 +1423,26 @@ void mr_launch_resolve_all(const ViewDev* views, int n_views, const uint64_t* pi
 }
 
 size_t mr_full_scratch_bytes() { return sizeof(uint32_t) * ((size_t)MR_FULL_CHUNK + 64); }
-uint64_t mr_full_chunk() { return MR_FULL_SPLIT ? MR_FULL_CHUNK : 0; }
+uint64_t mr_full_chunk() { return MR_FULL_CHUNK; }
+
+typedef void (*BackwardFn)(const SceneDev*, const ViewDev*, int, uint64_t, Rng, const float* const*, const GradDev*,
+                           const void*, int, unsigned long long*);
+
+template <bool DEMOD>
+static BackwardFn backward_fn(bool interp, bool packed)
+{
+    return interp ? (packed ? k_backward<true, DEMOD, true> : k_backward<true, DEMOD, false>)
+                  : (packed ? k_backward<false, DEMOD, true> : k_backward<false, DEMOD, false>);
+}
 
 void mr_launch_backward(const SceneDev* scenes, const ViewDev* views, int n_views, uint64_t total, Rng rng,
                         const float* const* d_images, const GradDev* grads, const void* tape,
                         unsigned long long* counters, int sms, cudaStream_t st, int nvx, void* full_scratch,
-                        bool interp)
+                        bool interp, bool packed)
 {
-#if MR_FULL_SPLIT
     // the primary vertex of every sample (the tape's FULL records are read by k_full only)
-    (interp ? k_backward<false, MR_BWD_MINB, true> : k_backward<false, MR_BWD_MINB, false>)<<<
-        grid_cap(total, 256, sms * 8), 256, 0, st>>>(scenes, views, n_views, total, rng, d_images, grads, tape, nvx,
-                                                     counters);
+    backward_fn<false>(interp, packed)<<<grid_cap(total, 256, sms * 8), 256, 0, st>>>(
+        scenes, views, n_views, total, rng, d_images, grads, tape, nvx, counters);
     if (nvx <= 0) return;
     unsigned int* bins = static_cast<unsigned int*>(full_scratch);  // [0, 16) counts, [16, 32) cursors, [32] total
     uint32_t* list = bins + 64;
@@ -1388,16 +1456,17 @@ void mr_launch_backward(const SceneDev* scenes, const ViewDev* views, int n_view
         k_full<<<grid, 256, 0, st>>>(scenes, views, n_views, total, rng, d_images, grads, tape, nvx, first, list, bins,
                                      n);
     }
-#else
-    (void)full_scratch;
-    (void)interp;
-    if (nvx > 0)
-        k_backward<true, MR_FULL_MINB, true><<<grid_cap(total, 256, sms * 8), 256, 0, st>>>(scenes, views, n_views, total, rng,
-                                                                          d_images, grads, tape, nvx, counters);
-    else
-        k_backward<false, MR_BWD_MINB, true><<<grid_cap(total, 256, sms * 8), 256, 0, st>>>(
-            scenes, views, n_views, total, rng, d_images, grads, tape, 0, counters);
-#endif
+}
+
+void mr_launch_tex_pack(const SceneDev* scenes, int n_scenes, uint64_t most_texels, int sms, cudaStream_t st)
+{
+    k_tex_pack<<<dim3(grid_cap(most_texels, 256, sms * 8), n_scenes), 256, 0, st>>>(scenes);
+}
+
+void mr_launch_grads_unpack(const SceneDev* scenes, const GradDev* grads, int n_scenes, uint64_t most, int sms,
+                            cudaStream_t st)
+{
+    k_grads_unpack<<<dim3(grid_cap(most, 256, sms * 8), n_scenes), 256, 0, st>>>(scenes, grads);
 }
 
 int mr_light_tile_pixels(int spp) { return spp <= LD_BLOCK ? LD_BLOCK / spp : 1; }
@@ -1414,11 +1483,10 @@ void mr_launch_light_demod(const SceneDev* scenes, const ViewDev* views, const u
 
 void mr_launch_light_backward(const SceneDev* scenes, const ViewDev* views, int n_views, uint64_t total, Rng rng,
                               const float* const* d_demod, const GradDev* grads, const void* tape,
-                              unsigned long long* counters, int sms, cudaStream_t st, bool interp)
+                              unsigned long long* counters, int sms, cudaStream_t st, bool interp, bool packed)
 {
-    (interp ? k_backward<false, MR_BWD_MINB, true, true> : k_backward<false, MR_BWD_MINB, false, true>)<<<
-        grid_cap(total, 256, sms * 8), 256, 0, st>>>(scenes, views, n_views, total, rng, d_demod, grads, tape, 0,
-                                                     counters);
+    backward_fn<true>(interp, packed)<<<grid_cap(total, 256, sms * 8), 256, 0, st>>>(
+        scenes, views, n_views, total, rng, d_demod, grads, tape, 0, counters);
 }
 
 void mr_launch_account(unsigned long long* counters, const unsigned int* qcnt, int bounces, uint64_t primary,

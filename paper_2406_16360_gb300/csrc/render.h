@@ -50,6 +50,11 @@ struct GradDev {
     float* metal;
     float* env;
     float* verts;
+    // packed accumulators of one call (null: none), added to the above by mr_launch_grads_unpack:
+    // per texel (albedo, roughness) (metallic, -), per env texel and per vertex (x, y, z, -)
+    float4* ptex;
+    float4* penv;
+    float4* pvert;
 };
 
 void mr_launch_raygen(const ViewDev& v, Rng rng, uint32_t first, uint32_t n, const QueueDev& q, void* tape,
@@ -83,11 +88,16 @@ void mr_launch_resolve_all(const ViewDev* views, int n_views, const uint64_t* pi
 // nvx = 0: PRIMARY-mode adjoint; nvx > 0: FULL mode over vertex records 1 .. nvx
 // scratch of the FULL-mode adjoint (per-class counts and one chunk's sample list), device bytes
 size_t mr_full_scratch_bytes();
-uint64_t mr_full_chunk();  // samples per FULL-mode pass (0: one kernel does every vertex)
+uint64_t mr_full_chunk();  // samples per FULL-mode pass
 void mr_launch_backward(const SceneDev* scenes, const ViewDev* views, int n_views, uint64_t total, Rng rng,
                         const float* const* d_images, const GradDev* grads, const void* tape,
                         unsigned long long* counters, int sms, cudaStream_t st, int nvx, void* full_scratch,
-                        bool interp);
+                        bool interp, bool packed);
+// packed: the scenes carry tex8 and the gradients their packed accumulators (zeroed)
+// (most: of any one scene's texels, resp. texels, env texels and vertices; n_scenes <= 65535)
+void mr_launch_tex_pack(const SceneDev* scenes, int n_scenes, uint64_t most_texels, int sms, cudaStream_t st);
+void mr_launch_grads_unpack(const SceneDev* scenes, const GradDev* grads, int n_scenes, uint64_t most, int sms,
+                            cudaStream_t st);
 void mr_launch_l2(const float* img, const float* ref, int64_t n, float* dimg, float* loss, int sms, cudaStream_t st);
 // monochrome light regulariser: the demodulated lighting per pixel (out[view] [h][w][4]) and
 // the PRIMARY-mode adjoint of it (d_demod[view] [h][w][3])
@@ -99,7 +109,7 @@ void mr_launch_light_demod(const SceneDev* scenes, const ViewDev* views, const u
                            cudaStream_t st, bool interp);
 void mr_launch_light_backward(const SceneDev* scenes, const ViewDev* views, int n_views, uint64_t total, Rng rng,
                               const float* const* d_demod, const GradDev* grads, const void* tape,
-                              unsigned long long* counters, int sms, cudaStream_t st, bool interp);
+                              unsigned long long* counters, int sms, cudaStream_t st, bool interp, bool packed);
 void mr_launch_trace_rays(const SceneDev& s, const float* rays, const int32_t* skip, int64_t n, int any,
                           int32_t* hit_tri, float* hit_tuv, int sms, cudaStream_t st);
 
