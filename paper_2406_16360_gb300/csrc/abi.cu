@@ -63,6 +63,11 @@ SceneDev mr_scene_dev(const mirres_scene* s)
     d.env_flat = s->env_flat;
     d.env_gflat = s->env_gflat;
     d.gf_shift = s->gf_shift;
+    d.ew_shift = 31;
+    while ((1ull << (d.ew_shift - 31)) < (unsigned long long)s->desc.env_w) ++d.ew_shift;
+    d.ew_mul = (uint32_t)(((1ull << d.ew_shift) + (unsigned long long)s->desc.env_w - 1) / (unsigned long long)s->desc.env_w);
+    d.env_dth = MR_PI / (float)s->desc.env_h;
+    d.env_dps = (2.0f * MR_PI) / (float)s->desc.env_w;
     d.n_tris = s->desc.n_tris;
     d.n_verts = s->desc.n_verts;
     d.tw = s->desc.tex_w;
