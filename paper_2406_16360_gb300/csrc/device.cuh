@@ -634,6 +634,21 @@ __device__ __forceinline__ float slab(float3 lo, float3 hi, float3 oi, float3 in
     return (tn <= tf * 1.0000005f + 1e-30f) ? tn : __int_as_float(0x7fffffff);
 }
 
+// The same test for the lane-refilling traversal: whether the ray meets the box at tn <= tmax. tmax is
+// compared behind the slack instead of in front of it (the same decision: rounding is monotone and
+// tmax >= 0), which leaves one comparison a box. Continuation rays 979 -> 932 us, shadow rays 1291 ->
+// 1197 us (ten-scene batch); one ray per thread ran 2% slower with it and keeps slab().
+__device__ __forceinline__ bool slab_hit(float3 lo, float3 hi, float3 oi, float3 inv, float tmin, float tmax,
+                                         float& tn)
+{
+    const float tx0 = fmaf(lo.x, inv.x, -oi.x), tx1 = fmaf(hi.x, inv.x, -oi.x);
+    const float ty0 = fmaf(lo.y, inv.y, -oi.y), ty1 = fmaf(hi.y, inv.y, -oi.y);
+    const float tz0 = fmaf(lo.z, inv.z, -oi.z), tz1 = fmaf(hi.z, inv.z, -oi.z);
+    tn = fmaxf(fmaxf(fminf(tx0, tx1), fminf(ty0, ty1)), fmaxf(fminf(tz0, tz1), tmin));
+    const float tf = fminf(fminf(fmaxf(tx0, tx1), fmaxf(ty0, ty1)), fmaxf(tz0, tz1));
+    return tn <= fminf(tf * 1.0000005f + 1e-30f, tmax);
+}
+
 // One traversal node (64 bytes, 64-byte aligned): the two child boxes and the child codes. With
 // MR_NODE_LD256 as two 32-byte loads (ld.global.nc.v8.f32, sm_100 and later) instead of four.
 __device__ __forceinline__ void load_node(const float4* p, float4& n0, float4& n1, float4& n2, int2& ch)
@@ -973,9 +988,9 @@ __device__ __forceinline__ void trav_warp(const SceneDev& s, Trav& T, uint32_t* 
                 float4 n0, n1, n2;
                 int2 ch;
                 load_node(T.nodes + 4 * (size_t)T.node, n0, n1, n2, ch);
-                const float tl = slab(f3(n0.x, n0.y, n0.z), f3(n0.w, n1.x, n1.y), T.oi, T.inv, T.tmin, T.best.t);
-                const float tr = slab(f3(n1.z, n1.w, n2.x), f3(n2.y, n2.z, n2.w), T.oi, T.inv, T.tmin, T.best.t);
-                bool gl = tl <= T.best.t, gr = tr <= T.best.t;
+                float tl, tr;
+                bool gl = slab_hit(f3(n0.x, n0.y, n0.z), f3(n0.w, n1.x, n1.y), T.oi, T.inv, T.tmin, T.best.t, tl);
+                bool gr = slab_hit(f3(n1.z, n1.w, n2.x), f3(n2.y, n2.z, n2.w), T.oi, T.inv, T.tmin, T.best.t, tr);
                 if (gl && ch.x < 0) {
                     sstk[(MR_SSTACK + T.pend) * sstride] = (uint32_t)~ch.x;
                     ++T.pend;
