@@ -159,31 +159,40 @@ __device__ __forceinline__ void shade_vertex(const SceneDev& s, int env_ok, cons
         int sel = -1, ytex = 0;
         uint32_t ysub = 0u;
         float3 ysel = f3(0.f, 0.f, 0.f);
+        // A candidate's weight and the lobe terms its colour is rebuilt from. Without a branch, so that the
+        // two candidates of a round are worked out side by side; what a direction below the horizon gives is
+        // dropped (about half of them are, but hardly ever all of a warp's). Shade stage 645 -> 627 us on
+        // config 2, 1840 -> 1822 us on a ten-scene batch.
+        struct Cand {
+            float ci, yfc, dv, w5;
+        };
+        auto weigh = [&](float3 dir) {
+            Cand c;
+            c.ci = dot(sh.n, dir);
+            const float3 h = normalize(add(wo, dir));
+            const float cnh = dot(sh.n, h), coh = dot(wo, h);
+            const float k = ggx_k(sh.n, h, cnh, a2);
+            const float D = __fdividef(a2, MR_PI * k * k);
+            c.dv = D * __fdividef(0.5f, c.ci * Ao + co * smith_a(a2, c.ci));
+            const float om = 1.0f - coh;
+            c.w5 = (om * om) * (om * om) * om;
+            const float yfc = (ykd + c.dv * (yf0 * (1.0f - c.w5) + c.w5)) * c.ci;  // Y(f_r) cos
+            c.yfc = (co > 0.0f && c.ci > 0.0f && above_face(sh, dir)) ? yfc : 0.0f;
+            return c;
+        };
         // candidate j with direction dir, texel tex and gq = Y(L_env) / q_dir into the reservoir
-        auto consider = [&](int j, const uint4& x, float3 dir, int tex, float gq) {
-            const float ci = dot(sh.n, dir);
-            float yfc = 0.0f, dv = 0.0f, w5 = 0.0f;
-            if (co > 0.0f && ci > 0.0f && above_face(sh, dir)) {
-                const float3 h = normalize(add(wo, dir));
-                const float cnh = dot(sh.n, h), coh = dot(wo, h);
-                const float k = ggx_k(sh.n, h, cnh, a2);
-                const float D = __fdividef(a2, MR_PI * k * k);
-                dv = D * __fdividef(0.5f, ci * Ao + co * smith_a(a2, ci));
-                const float om = 1.0f - coh;
-                w5 = (om * om) * (om * om) * om;
-                yfc = (ykd + dv * (yf0 * (1.0f - w5) + w5)) * ci;  // Y(f_r) cos
-            }
-            const float gamma = yfc * gq;  // gamma = p_hat / q_dir, p_hat = Y(L_env) Y(f_r) cos
+        auto consider = [&](int j, const uint4& x, float3 dir, int tex, float gq, const Cand& c) {
+            const float gamma = c.yfc * gq;  // gamma = p_hat / q_dir, p_hat = Y(L_env) Y(f_r) cos
             wsum += gamma;
             if (u24(x.z) * wsum < gamma) {
                 sel = j;
                 ytex = tex;
                 ysub = x.w;
                 ysel = dir;
-                yfc_sel = yfc;
-                dv_sel = dv;
-                w5_sel = w5;
-                ci_sel = ci;
+                yfc_sel = c.yfc;
+                dv_sel = c.dv;
+                w5_sel = c.w5;
+                ci_sel = c.ci;
             }
         };
         int j = 0;
@@ -199,8 +208,9 @@ __device__ __forceinline__ void shade_vertex(const SceneDev& s, int env_ok, cons
             float4 rv0, rv1;
             const float st0 = env_dir(s, r0, c0, x0.w, d0, rv0);
             const float st1 = env_dir(s, r1, c1, x1.w, d1, rv1);
-            consider(j, x0, d0, r0 * s.ew + c0, st0 * rv0.z);
-            consider(j + 1, x1, d1, r1 * s.ew + c1, st1 * rv1.z);
+            const Cand e0 = weigh(d0), e1 = weigh(d1);
+            consider(j, x0, d0, r0 * s.ew + c0, st0 * rv0.z, e0);
+            consider(j + 1, x1, d1, r1 * s.ew + c1, st1 * rv1.z, e1);
         }
 #endif
 #pragma unroll kCandUnroll
@@ -209,7 +219,7 @@ __device__ __forceinline__ void shade_vertex(const SceneDev& s, int env_ok, cons
             float3 dir;
             int tex;
             const float gq = env_candidate(s, x.x, x.y, x.w, dir, tex);
-            consider(j, x, dir, tex, gq);
+            consider(j, x, dir, tex, gq, weigh(dir));
         }
         const float4 L = (sel >= 0) ? __ldg(s.env_texel + ytex) : make_float4(0.f, 0.f, 0.f, 0.f);
         const float phat_sel = lum(xyz(L)) * yfc_sel;
