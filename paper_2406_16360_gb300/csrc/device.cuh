@@ -100,7 +100,7 @@ struct SceneDev {
     const float2* env_col;    // [ew]: (cos psi_c, sin psi_c), psi = 2 pi u - pi at column centres
     int32_t env_fine;         // 1 when a texel spans at most pi/32 in both angles (tables used)
     const unsigned long long* env_flat; // [eh ew + 1] ceil(cdf 2^53) of the CDF over all texels
-    const uint32_t* env_gflat;          // [gf + 1] guide: answer of the search at bucket starts
+    const uint32_t* env_gflat;          // [gf + 1] guide: answer of the search at bucket starts (bits 0-30)
     int32_t gf_shift;
     // row of a texel index by a multiplication (row_of_texel), and the angles of a texel: pi / eh
     // and 2 pi / ew
@@ -295,6 +295,10 @@ __device__ __forceinline__ float env_dir(const SceneDev& s, int r, int c, uint32
 // searches start from guide tables (cut-point method): the answer at the start of the
 // uniform's bucket and at the next bucket bound the answer, so the search is the same
 // function of the uniform as a full binary search, over a range of ~1-2 entries.
+// Bit 31 of a guide entry says that the next entry differs; without it the search is over (88% of the
+// draws on a 1024 x 512 env with a sun) and the next entry is not read: shade stage 1840 -> 1827 us on
+// a ten-scene batch, 382 -> 372 us on a 120k-triangle step.
+constexpr uint32_t GUIDE_MORE = 0x80000000u;
 // the texel of the CDF over all texels (row-major) at the 53-bit uniform k 2^-53,
 // k = xa 2^21 + (xb >> 11): the largest t with threshold[t] <= k, searched inside the range
 // the guide gives for k's bucket
@@ -302,7 +306,9 @@ __device__ __forceinline__ void env_texel_draw(const SceneDev& s, uint32_t xa, u
 {
     const unsigned long long k = ((unsigned long long)xa << 21) | (unsigned long long)(xb >> 11);
     const uint32_t b = (uint32_t)(k >> s.gf_shift);
-    int lo = (int)__ldg(s.env_gflat + b), hi = (int)__ldg(s.env_gflat + b + 1);
+    const uint32_t e = __ldg(s.env_gflat + b);
+    int lo = (int)(e & ~GUIDE_MORE), hi = lo;
+    if (e & GUIDE_MORE) hi = (int)(__ldg(s.env_gflat + b + 1) & ~GUIDE_MORE);
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
         if (__ldg(s.env_flat + mid) <= k) lo = mid;
@@ -320,8 +326,10 @@ __device__ __forceinline__ void env_texel_draw2(const SceneDev& s, uint32_t xa0,
     const unsigned long long k0 = ((unsigned long long)xa0 << 21) | (unsigned long long)(xb0 >> 11);
     const unsigned long long k1 = ((unsigned long long)xa1 << 21) | (unsigned long long)(xb1 >> 11);
     const uint32_t b0 = (uint32_t)(k0 >> s.gf_shift), b1 = (uint32_t)(k1 >> s.gf_shift);
-    int lo0 = (int)__ldg(s.env_gflat + b0), hi0 = (int)__ldg(s.env_gflat + b0 + 1);
-    int lo1 = (int)__ldg(s.env_gflat + b1), hi1 = (int)__ldg(s.env_gflat + b1 + 1);
+    const uint32_t e0 = __ldg(s.env_gflat + b0), e1 = __ldg(s.env_gflat + b1);
+    int lo0 = (int)(e0 & ~GUIDE_MORE), lo1 = (int)(e1 & ~GUIDE_MORE), hi0 = lo0, hi1 = lo1;
+    if (e0 & GUIDE_MORE) hi0 = (int)(__ldg(s.env_gflat + b0 + 1) & ~GUIDE_MORE);
+    if (e1 & GUIDE_MORE) hi1 = (int)(__ldg(s.env_gflat + b1 + 1) & ~GUIDE_MORE);
     while (lo0 < hi0 || lo1 < hi1) {
         const int m0 = (lo0 + hi0 + 1) >> 1, m1 = (lo1 + hi1 + 1) >> 1;
         const bool a0 = lo0 < hi0, a1 = lo1 < hi1;

@@ -223,7 +223,10 @@ __global__ void __launch_bounds__(256) k_env_flat_guide(const unsigned long long
         if (b == g) t = n - 1;
         else if (staged) t = t0 + search_in(s, 0, m - 1, k);
         else t = search_in(flat, 0, n - 1, k);
-        guide[b] = (uint32_t)t;
+        // the bucket's answer may be a later texel: the next threshold is reached before the next bucket
+        const unsigned long long next = (unsigned long long)(b + 1) << shift;
+        const bool more = t + 1 < n && (staged && t + 1 - t0 < m ? s[t + 1 - t0] : flat[t + 1]) <= next;
+        guide[b] = (uint32_t)t | (more ? GUIDE_MORE : 0u);
     }
 }
 

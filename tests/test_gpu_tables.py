@@ -81,3 +81,33 @@ def test_env_tables_at_chunk_edges(M, ctx, ew, eh, sun):  # noqa: F811
     for s in gw.scenes:
         s.close()
     ds.close()
+
+
+@pytest.mark.parametrize("ew,eh", [(64, 32), (67, 33), (3, 1)])
+def test_guide_over_black_texels(M, ctx, ew, eh):  # noqa: F811
+    """rows and runs of black texels (equal thresholds, which a guide bucket may hold many of, or whose
+    next entry lies far on): the draws of a render are those of a search over all thresholds"""
+    from paper_2406_16360_gb300.renderer import GpuWorkload
+    rng = np.random.Generator(np.random.PCG64(ew))
+    sc = synth.tiny_scene(subdiv=1)
+    sc.env = rng.uniform(0.1, 2.0, size=(eh, ew, 3)).astype(np.float32)
+    sc.env[1:eh // 3] = 0.0
+    sc.env[:, ew // 4:ew // 2] = 0.0
+    sc.env[0, 0] = 1e-6  # a sliver of a bucket before the next threshold
+    K, c2w = synth.look_at((0.0, 1.5, 4.0), (0.0, 1.0, 0.0), 64, 48, 40.0)
+    w = synth.Workload("env", [sc], [synth.View(K, c2w, 64, 48, 4, 1)], ris_m=9, seed=2)
+    gw = GpuWorkload(w, 0, ctx=ctx)
+    flat = torch.zeros(eh * ew + 1, dtype=torch.int64, device="cuda")
+    M.mirres_env_export_flat(gw.scenes[0].handle, flat)
+    _, tape = gw.render(launch=1)
+    torch.cuda.synchronize()
+    words = tape.cpu().numpy().reshape(-1, w.samples)
+    cand, ytex = words[1], words[9]
+    g = np.flatnonzero(cand >= 0)
+    assert len(g)
+    x = philox4x32_10(g // 4, g % 4, np.full_like(g, 1), cand[g], w.seed, 0)
+    k = (x[0].astype(np.uint64) << np.uint64(21)) | (x[1].astype(np.uint64) >> np.uint64(11))
+    want = np.searchsorted(flat.cpu().numpy().view(np.uint64), k, side="right") - 1
+    assert np.array_equal(ytex[g], want)
+    for s in gw.scenes:
+        s.close()
