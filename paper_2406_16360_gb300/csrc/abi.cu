@@ -230,6 +230,7 @@ extern "C" mirres_status mirres_context_destroy(mirres_context* ctx)
     cudaSetDevice(ctx->device);
     cudaDeviceSynchronize();
     if (ctx->graph) cudaGraphExecDestroy(ctx->graph);
+    if (ctx->graph_src) cudaGraphDestroy(ctx->graph_src);
     for (int i = 0; i < ctx->n_stage_events; ++i) cudaEventDestroy(ctx->stage_events[i]);
     delete[] ctx->stage_events;
     delete[] ctx->stage_kind;
@@ -623,11 +624,32 @@ static mirres_status render_wave(mirres_context* ctx, const std::vector<SceneDev
     key.ws_bytes = ctx->ws.bytes;
     key.shape = ctx->wave_shape;
     static_assert(sizeof(GraphKey) <= sizeof(ctx->graph_key), "graph key too large");
+    GraphKey have;
+    std::memcpy(&have, ctx->graph_key, sizeof(have));
+    if (ctx->graph && (have.k0 != key.k0 || have.k1 != key.k1)) {
+        // every step of an optimisation loop has a seed of its own: when nothing else differs the keys
+        // are replaced in the captured graph (a capture and instantiation takes some 100 us on the host)
+        have.k0 = key.k0;
+        have.k1 = key.k1;
+        if (std::memcmp(&have, &key, sizeof(key)) == 0) {
+            if (mr_wave_reseed(ctx->graph, ctx->seeded, rng) == cudaSuccess) {
+                std::memcpy(ctx->graph_key, &key, sizeof(key));
+            } else {
+                cudaGetLastError();
+                std::memset(ctx->graph_key, 0, sizeof(ctx->graph_key));  // partly rewritten: captured again
+            }
+        }
+    }
     if (!ctx->graph || std::memcmp(ctx->graph_key, &key, sizeof(key)) != 0) {
         if (ctx->graph) {
             cudaGraphExecDestroy(ctx->graph);
             ctx->graph = nullptr;
         }
+        if (ctx->graph_src) {
+            cudaGraphDestroy(ctx->graph_src);
+            ctx->graph_src = nullptr;
+        }
+        ctx->seeded.count = 0;
         if (!ctx->capture_stream) MR_CUDA(cudaStreamCreateWithFlags(&ctx->capture_stream, cudaStreamNonBlocking));
         br[0].st = ctx->capture_stream;
         for (int b = 0; b < nb; ++b) {
@@ -645,7 +667,7 @@ static mirres_status render_wave(mirres_context* ctx, const std::vector<SceneDev
                        ctx->sm_count, (flags & 1) ? ctx->stage_events : nullptr,
                        (flags & 1) ? ctx->stage_kind : nullptr, nvx, (flags & 2) != 0, reuse_k, reuse_radius, res,
                        temporal, temporal_cap, hist, vdev.data(), sdev.data(), (flags & 4) != 0, bin,
-                       ctx->wave_shape);
+                       ctx->wave_shape, &ctx->seeded);
         ctx->stage_pairs = (flags & 1) ? pairs : 0;
         cudaGraph_t g = nullptr;
         const cudaError_t ec = cudaStreamEndCapture(ctx->capture_stream, &g);
@@ -654,11 +676,12 @@ static mirres_status render_wave(mirres_context* ctx, const std::vector<SceneDev
             return mr_cuda_status(ec, "mirres_render: graph capture");
         }
         const cudaError_t ei = cudaGraphInstantiate(&ctx->graph, g, 0);
-        cudaGraphDestroy(g);
         if (ei != cudaSuccess) {
+            cudaGraphDestroy(g);
             ctx->graph = nullptr;
             return mr_cuda_status(ei, "mirres_render: graph instantiation");
         }
+        ctx->graph_src = g;
         std::memcpy(ctx->graph_key, &key, sizeof(key));
         int raster_launches = 0;
         if (flags & 4) {

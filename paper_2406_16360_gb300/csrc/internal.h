@@ -30,6 +30,15 @@ enum { CNT_PRIMARY = 0, CNT_CONT, CNT_SHADOW, CNT_SAMPLES, CNT_DIFF, CNT_CAND, C
        // rays, then of shadow rays
        CNT_CBOX, CNT_CTRI, CNT_SBOX, CNT_STRI, CNT_N };
 
+// the kernel nodes of a captured forward whose third argument is the seed's round keys (count < 0: not
+// known, or more than fit, as with over a hundred waves)
+struct SeededNodes {
+    enum { MAX = 512, MAX_ARGS = 20 };
+    int count = 0;
+    cudaGraphNode_t node[MAX];
+    int n_args[MAX];
+};
+
 struct mirres_context {
     int device = 0;
     int sm_count = 0;
@@ -43,6 +52,8 @@ struct mirres_context {
     // batched wavefront: the captured forward and the arguments it was captured for
     cudaStream_t capture_stream = nullptr;
     cudaGraphExec_t graph = nullptr;
+    cudaGraph_t graph_src = nullptr;         // what it was instantiated from, for its seeded nodes
+    SeededNodes seeded;
     unsigned char graph_key[192] = {};
     mirres_wave_shape wave_shape = {25, {256, 256, 256, 256}, {8, 8, 8, 8}, 1};  // batched wavefront launch shape
     cudaStream_t branch_stream[4] = {};  // [1..3]: the streams of wave chains 1..3 during capture

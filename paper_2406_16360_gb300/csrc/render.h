@@ -154,6 +154,7 @@ void mr_wave_record(const SceneDev* scenes, const ViewDev* views, int n_views, u
                     const uint64_t* pix_off, uint64_t total_pix, float* const* images, int sms, cudaEvent_t* ev,
                     int* kind, int nvx, bool count, int reuse_k, int reuse_radius, const ResDev& res, int temporal,
                     int temporal_cap, const HistDev& hist, const ViewDev* hviews, const SceneDev* hscenes, bool raster,
-                    bool bin, const mirres_wave_shape& shape);
+                    bool bin, const mirres_wave_shape& shape, SeededNodes* seeded);
+cudaError_t mr_wave_reseed(cudaGraphExec_t exec, const SeededNodes& nodes, Rng rng);
 int mr_wave_launches(int n_waves, int max_bounces, bool reuse, int temporal, int raster_launches, bool bin);
 int mr_wave_stage_pairs(int n_waves, int max_bounces);

@@ -799,6 +799,27 @@ __global__ void __launch_bounds__(256) k_raster_big(const SceneDev* __restrict__
     }
 }
 
+// The kernel node just captured on `st`, whose third argument is the random numbers' keys, onto the list
+// of nodes a call with another seed rewrites. With anything unexpected about the capture the list is
+// marked as unusable (count < 0) and such a call captures again.
+template <class... A>
+void keep_seeded(cudaStream_t st, void (*)(A...), SeededNodes* out)
+{
+    if (!out || out->count < 0) return;
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    const cudaGraphNode_t* deps = nullptr;
+    size_t n = 0;
+    cudaGraphNodeType type = cudaGraphNodeTypeEmpty;
+    if (cudaStreamGetCaptureInfo(st, &status, nullptr, nullptr, &deps, nullptr, &n) != cudaSuccess ||
+        status != cudaStreamCaptureStatusActive || n != 1 || cudaGraphNodeGetType(deps[0], &type) != cudaSuccess ||
+        type != cudaGraphNodeTypeKernel || sizeof...(A) > SeededNodes::MAX_ARGS || out->count >= SeededNodes::MAX) {
+        out->count = -1;
+        return;
+    }
+    out->node[out->count] = deps[0];
+    out->n_args[out->count++] = (int)sizeof...(A);
+}
+
 unsigned grid_cap(uint64_t n, int block, int cap)
 {
     const uint64_t g = (n + block - 1) / block;
@@ -816,7 +837,7 @@ void mr_wave_record(const SceneDev* scenes, const ViewDev* views, int n_views, u
                     const uint64_t* pix_off, uint64_t total_pix, float* const* images, int sms, cudaEvent_t* ev,
                     int* kind, int nvx, bool count, int reuse_k, int reuse_radius, const ResDev& res, int temporal,
                     int temporal_cap, const HistDev& hist, const ViewDev* hviews, const SceneDev* hscenes, bool raster,
-                    bool bin, const mirres_wave_shape& shape)
+                    bool bin, const mirres_wave_shape& shape, SeededNodes* seeded)
 {
     // waves go round-robin to `n_branches` chains of their own (queues, counters, stream): chain
     // 0 on the recording stream, the others forked from it and joined back before the resolve,
@@ -866,6 +887,7 @@ void mr_wave_record(const SceneDev* scenes, const ViewDev* views, int n_views, u
         mark(3, true);
         k_wraygen<<<grid_cap(n, blk_g, cap_g), blk_g, 0, st>>>(views, n_views, rng, first, n, qa, tape, total, nvx,
                                                                res);
+        keep_seeded(st, k_wraygen, seeded);
         mark(3, false);
         QueueDev cur = qa, nxt = qb;
         for (int b = 0; b < max_bounces; ++b) {
@@ -919,12 +941,17 @@ void mr_wave_record(const SceneDev* scenes, const ViewDev* views, int n_views, u
                      : (interp ? k_wshade<false, true> : k_wshade<false, false>))<<<grid_cap(n, blk_h, cap_h), blk_h, 0, st>>>(
                 scenes, views, rng, b, M, hq, qc + 3 * b, nxt, qc + 3 * b + 1, sq, qc + 3 * b + 2, tape, total, nvx,
                 res, counters);
-            if (reuse_b && temporal == 2)
+            keep_seeded(st, k_wshade<false, false>, seeded);
+            if (reuse_b && temporal == 2) {
                 k_wtemporal<<<grid_cap(n, blk_h, cap_h), blk_h, 0, st>>>(scenes, views, rng, M, temporal_cap, hq, qc,
                                                                          res, hist);
-            if (reuse_b)
+                keep_seeded(st, k_wtemporal, seeded);
+            }
+            if (reuse_b) {
                 k_wreuse<<<grid_cap(n, blk_h, cap_h), blk_h, 0, st>>>(scenes, views, rng, M, reuse_k, reuse_radius, hq,
                                                                       qc, sq, qc + 2, res, hist, tape, total, nvx);
+                keep_seeded(st, k_wreuse, seeded);
+            }
             if (reuse_b && temporal)
                 k_whist_miss<<<grid_cap(n, blk_h, cap_h), blk_h, 0, st>>>(first, n, tape, total, hist);
             mark(1, false);
@@ -948,6 +975,26 @@ void mr_wave_record(const SceneDev* scenes, const ViewDev* views, int n_views, u
         cudaStreamWaitEvent(st_main, join[b], 0);
     }
     mr_launch_resolve_all(views, n_views, pix_off, total_pix, images, tape, total, sms, st_main);
+}
+
+// New keys for a captured forward: the argument of its seeded kernels, a microsecond or two a node. The
+// launches already made keep theirs.
+cudaError_t mr_wave_reseed(cudaGraphExec_t exec, const SeededNodes& nodes, Rng rng)
+{
+    if (nodes.count < 0) return cudaErrorInvalidValue;
+    for (int i = 0; i < nodes.count; ++i) {
+        cudaKernelNodeParams p{};
+        cudaError_t e = cudaGraphKernelNodeGetParams(nodes.node[i], &p);
+        if (e != cudaSuccess) return e;
+        if (!p.kernelParams || p.extra) return cudaErrorInvalidValue;
+        void* args[SeededNodes::MAX_ARGS];
+        for (int k = 0; k < nodes.n_args[i]; ++k) args[k] = p.kernelParams[k];
+        args[2] = &rng;
+        p.kernelParams = args;
+        e = cudaGraphExecKernelNodeSetParams(exec, nodes.node[i], &p);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 int mr_wave_stage_pairs(int n_waves, int max_bounces) { return n_waves * (1 + 3 * max_bounces); }
