@@ -77,3 +77,32 @@ def test_put_aside_leaves_change_nothing(M, ctx, mesh, width, height, spp, bounc
     assert capped[0] == capped[1] and (cap > 0 or capped[0] == 0)
     for s in gw.scenes:
         s.close()
+
+
+@pytest.mark.parametrize("mesh", ["shells", "funnel", "one"])
+@pytest.mark.parametrize("n", [1, 31, 33, 257, 400001])
+def test_ray_queries_do_not_depend_on_their_neighbours(M, ctx, mesh, n):
+    """lanes refilled from runs of 32 rays (400,001: more than one round of the grid): every ray's answer
+    is the one it gets in another order, and any hit agrees with closest hit"""
+    from paper_2406_16360_gb300.renderer import GpuWorkload
+    gw = GpuWorkload(_workload(mesh, 8, 8, 1, 1), 0, ctx=ctx)
+    h = gw.scenes[0].handle
+    g = torch.Generator(device="cuda").manual_seed(n)
+    o = torch.randn((n, 3), device="cuda", generator=g)
+    d = 0.8 * torch.randn((n, 3), device="cuda", generator=g) - o
+    rays = torch.cat([o, d / d.norm(dim=1, keepdim=True)], 1).contiguous()
+    skip = torch.randint(-1, 3, (n,), device="cuda", generator=g, dtype=torch.int32)
+    order = torch.randperm(n, device="cuda", generator=g)
+    out = []
+    for r, s in ((rays, skip), (rays[order].contiguous(), skip[order].contiguous())):
+        tri, any_ = (torch.full((n,), -7, device="cuda", dtype=torch.int32) for _ in range(2))
+        tuv = torch.full((n, 3), -7.0, device="cuda")
+        M.mirres_trace(ctx, h, r, tri, tuv, skip=s)
+        M.mirres_trace(ctx, h, r, any_, skip=s, any_hit=True)
+        torch.cuda.synchronize()
+        assert torch.equal(any_, torch.where(tri >= 0, 1, -1).to(torch.int32))
+        out.append((tri, tuv))
+    assert torch.equal(out[0][0][order], out[1][0]) and torch.equal(out[0][1][order], out[1][1])
+    assert n < 31 or int((out[0][0] >= 0).sum()) > 0
+    for s in gw.scenes:
+        s.close()
