@@ -685,6 +685,7 @@ static mirres_status render_wave(mirres_context* ctx, const std::vector<SceneDev
         std::memcpy(ctx->graph_key, &key, sizeof(key));
         int raster_launches = 0;
         if (flags & 4) {
+            raster_launches = n_waves;  // the rays the rasteriser reads
             for (int wv = 0; wv < n_waves; ++wv) {
                 const uint64_t f0 = wave_first[(size_t)wv];
                 const uint64_t f1 = wv + 1 < n_waves ? wave_first[(size_t)wv + 1] : total;

@@ -1,6 +1,6 @@
 // wave.cu -- batched wavefront: every view of every scene flattened into one sample space and
-// processed in large waves (ray generation, then per bounce: closest hit with hit compaction,
-// shading with RIS, shadow rays). Stage kernels are grid-stride loops over device-side queue
+// processed in large waves (per bounce: closest hit with hit compaction -- bounce 0 makes its camera
+// rays itself --, shading with RIS, shadow rays). Stage kernels are grid-stride loops over device-side queue
 // counts, so the whole forward is one fixed launch sequence that is captured once as a CUDA
 // graph and replayed. Each queued path carries its view index (in the w component of its
 // throughput), through which it finds its camera, spp, bounce count and scene.
@@ -8,6 +8,10 @@
 #include "render.h"
 
 namespace {
+
+// The throughput of L_ind is one at every vertex before this bounce: it is neither stored with the rays
+// and hits that lead there nor read.
+constexpr int BI_FROM = 2;
 
 // per-warp flush of a traversal stage's box and triangle test counts (counters idx, idx + 1)
 __device__ __forceinline__ void flush_work(unsigned long long* counters, int idx, unsigned int box, unsigned int tri)
@@ -20,47 +24,50 @@ __device__ __forceinline__ void flush_work(unsigned long long* counters, int idx
     }
 }
 
-__global__ void __launch_bounds__(256) k_wraygen(const ViewDev* __restrict__ views, int n_views, Rng rng,
-                                                 uint64_t first, uint32_t n, QueueDev q, void* tape, uint64_t ntot,
-                                                 int nvx, ResDev res)
+// the camera ray of the call's sample g: its view's index, its number in the view and its direction
+__device__ __forceinline__ const ViewDev& camera_ray(const ViewDev* views, int n_views, const Rng& rng, uint64_t g,
+                                                     int& vi, uint32_t& sid, float3& d)
 {
-    const TapeDev tp = tape_of(tape, ntot, nvx);
+    const ViewDev& v = view_of(views, n_views, g, vi);
+    sid = (uint32_t)(g - v.offset);
+    const uint32_t pixel = sid / (uint32_t)v.spp, smp = sid % (uint32_t)v.spp;
+    const int px = (int)(pixel % (uint32_t)v.width), py = (int)(pixel / (uint32_t)v.width);
+    const uint4 x = rng.draw(pixel, smp, (uint32_t)v.index, 0u, PURPOSE_CAMERA, 0u);
+    d = camera_dir(v, px, py, u24(x.x), u24(x.y));
+    return v;
+}
+
+// camera rays into a queue, for the rasteriser (otherwise the primary closest-hit kernel makes them)
+__global__ void __launch_bounds__(256) k_wraygen(const ViewDev* __restrict__ views, int n_views, Rng rng,
+                                                 uint64_t first, uint32_t n, QueueDev q)
+{
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const uint64_t g = first + i;
         int vi;
-        const ViewDev& v = view_of(views, n_views, g, vi);
-        const uint32_t sid = (uint32_t)(g - v.offset);
-        const uint32_t pixel = sid / (uint32_t)v.spp, smp = sid % (uint32_t)v.spp;
-        const int px = (int)(pixel % (uint32_t)v.width), py = (int)(pixel / (uint32_t)v.width);
-        const uint4 x = rng.draw(pixel, smp, (uint32_t)v.index, 0u, PURPOSE_CAMERA, 0u);
-        const float3 d = camera_dir(v, px, py, u24(x.x), u24(x.y));
+        uint32_t sid;
+        float3 d;
+        const ViewDev& v = camera_ray(views, n_views, rng, first + i, vi, sid, d);
         q.o[i] = make_float4(v.c2w[3], v.c2w[7], v.c2w[11], __int_as_float(-1));
         q.d[i] = make_float4(d.x, d.y, d.z, __uint_as_float(sid));
         q.b[i] = make_float4(1.f, 1.f, 1.f, __int_as_float(vi));
-        q.bi[i] = make_float4(1.f, 1.f, 1.f, 0.f);
-        tp.tri[g] = -1;
-        tp.cand[g] = -1;
-        tp.wv[g] = 0.0f;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            tp.lind[k][g] = 0.0f;
-            tp.rad[k][g] = 0.0f;
-        }
-        tape_vx_init(tp, g);
-        if (res.ytex) res.ytex[g] = RES_MISS;
     }
 }
 
-template <bool COUNT, bool RASTER, bool WIDE>
+// Closest hits, one ray per thread. PRIMARY: bounce 0, which makes its camera rays itself (those the
+// rasteriser resolves come from the queue) and starts their tape words: a separate ray generation wrote
+// 100 bytes a sample and this stage read 64 of them back, a millisecond of a 1920 x 1080 render at 32
+// samples that DRAM alone bounded (39.4 -> 38.0 ms; ten-scene batch 4.73 -> 4.59 ms).
+template <bool COUNT, bool RASTER, bool WIDE, bool PRIMARY>
 __global__ void MR_TRACE_BOUNDS k_wclosest(const SceneDev* __restrict__ scenes,
-                                                  const ViewDev* __restrict__ views, int b, QueueDev q,
-                                                  const unsigned int* count, unsigned int count_fixed, QueueDev hq,
-                                                  unsigned int* count_hit, void* tape, uint64_t ntot,
+                                                  const ViewDev* __restrict__ views, Rng rng, int n_views, int b,
+                                                  QueueDev q, uint64_t first, const unsigned int* count,
+                                                  unsigned int count_fixed, QueueDev hq, unsigned int* count_hit,
+                                                  void* tape, uint64_t ntot, int nvx, ResDev res,
                                                   unsigned long long* counters, const unsigned long long* raster)
 {
+    static_assert(PRIMARY || !RASTER, "only primary rays are rasterised");
     extern __shared__ __align__(16) uint32_t sstk[];
-    const TapeDev tp = tape_of(tape, ntot);
-    const unsigned int n = count ? *count : count_fixed;
+    const TapeDev tp = tape_of(tape, ntot, nvx);
+    const unsigned int n = PRIMARY ? count_fixed : *count;
     unsigned int n_box = 0;
     int n_tri = 0;
     const unsigned int stride = gridDim.x * blockDim.x;
@@ -71,9 +78,20 @@ __global__ void MR_TRACE_BOUNDS k_wclosest(const SceneDev* __restrict__ scenes,
         h.tri = -1;
         float4 qd = make_float4(0.f, 0.f, 0.f, 0.f), qb = qd;
         if (i < n) {
-            const float4 a = q.o[i];
-            qd = q.d[i];
-            qb = q.b[i];
+            float4 a;
+            if (PRIMARY && !RASTER) {
+                int vi;
+                uint32_t sid;
+                float3 d;
+                const ViewDev& v = camera_ray(views, n_views, rng, first + i, vi, sid, d);
+                a = make_float4(v.c2w[3], v.c2w[7], v.c2w[11], __int_as_float(-1));
+                qd = make_float4(d.x, d.y, d.z, __uint_as_float(sid));
+                qb = make_float4(1.f, 1.f, 1.f, __int_as_float(vi));
+            } else {
+                a = q.o[i];
+                qd = q.d[i];
+                qb = q.b[i];
+            }
             const ViewDev& v = views[__float_as_int(qb.w)];
             const SceneDev& s = scenes[v.scene];
             if (RASTER) {
@@ -104,12 +122,22 @@ __global__ void MR_TRACE_BOUNDS k_wclosest(const SceneDev* __restrict__ scenes,
                                           __int_as_float(0x7f800000), h, sstk + threadIdx.x);
                 }
             }
-            if (h.tri < 0 && b == 0) {
-                const uint64_t g = v.offset + __float_as_uint(qd.w);
-                const float4 L = __ldg(s.env_texel + env_texel_of(s, xyz(qd)));
+            if (PRIMARY) {  // the sample's tape words (shading writes the others of a hit)
+                const uint64_t g = first + i;
+                float4 L = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (h.tri < 0) {
+                    L = __ldg(s.env_texel + env_texel_of(s, xyz(qd)));
+                    tp.tri[g] = -1;
+                    tp.cand[g] = -1;
+                    tp.wv[g] = 0.0f;
+                    if (res.ytex) res.ytex[g] = RES_MISS;
+                }
                 tp.rad[0][g] = L.x;
                 tp.rad[1][g] = L.y;
                 tp.rad[2][g] = L.z;
+#pragma unroll
+                for (int k = 0; k < 3; ++k) tp.lind[k][g] = 0.0f;
+                tape_vx_init(tp, g);
             }
         }
         const bool hit = h.tri >= 0;
@@ -118,7 +146,7 @@ __global__ void MR_TRACE_BOUNDS k_wclosest(const SceneDev* __restrict__ scenes,
             hq.o[slot] = make_float4(h.t, h.u, h.v, __int_as_float(h.tri));
             hq.d[slot] = qd;
             hq.b[slot] = qb;
-            hq.bi[slot] = q.bi[i];
+            if (b >= BI_FROM) hq.bi[slot] = q.bi[i];
         }
     }
     if (COUNT) flush_work(counters, CNT_CBOX, n_box, (unsigned int)n_tri);
@@ -271,7 +299,7 @@ __global__ void __launch_bounds__(256, MR_SHADE_MINB) k_wshade(const SceneDev* _
             h.tri = tri;
             const int env_ok = *s.env_ok_dev;
             shade_vertex<INTERP>(s, env_ok, rng, pixel, smp, (uint32_t)v.index, b, v.bounces, M, h, xyz(qd), xyz(qb),
-                         xyz(hq.bi[i]), out);
+                         b >= BI_FROM ? xyz(hq.bi[i]) : f3(1.f, 1.f, 1.f), out);
             if (env_ok) n_cand += (unsigned long long)M;
             if (b == 0) {
                 tp.tri[g] = tri;
@@ -297,14 +325,14 @@ __global__ void __launch_bounds__(256, MR_SHADE_MINB) k_wshade(const SceneDev* _
             sq.o[ss] = make_float4(out.sh_o.x, out.sh_o.y, out.sh_o.z, __int_as_float(tri));
             sq.d[ss] = make_float4(out.sh_d.x, out.sh_d.y, out.sh_d.z, __uint_as_float(sid));
             sq.add[ss] = make_float4(out.add_rad.x, out.add_rad.y, out.add_rad.z, __int_as_float(vi));
-            sq.addi[ss] = make_float4(out.add_lind.x, out.add_lind.y, out.add_lind.z, 0.f);
+            if (b >= 1) sq.addi[ss] = make_float4(out.add_lind.x, out.add_lind.y, out.add_lind.z, 0.f);
         }
         const unsigned int cs = warp_append(out.cont, count_out);
         if (out.cont) {
             qout.o[cs] = make_float4(out.x.x, out.x.y, out.x.z, __int_as_float(tri));
             qout.d[cs] = make_float4(out.c_d.x, out.c_d.y, out.c_d.z, __uint_as_float(sid));
             qout.b[cs] = make_float4(out.c_beta.x, out.c_beta.y, out.c_beta.z, __int_as_float(vi));
-            qout.bi[cs] = make_float4(out.c_bind.x, out.c_bind.y, out.c_bind.z, 0.f);
+            if (b + 1 >= BI_FROM) qout.bi[cs] = make_float4(out.c_bind.x, out.c_bind.y, out.c_bind.z, 0.f);
         }
     }
     for (int off = 16; off > 0; off >>= 1) n_cand += __shfl_xor_sync(MR_FULL, n_cand, off);
@@ -337,11 +365,11 @@ __global__ void __launch_bounds__(256) k_wshadow(const SceneDev* __restrict__ sc
         }
         const uint64_t g = v.offset + __float_as_uint(dd.w);
         if (h.tri < 0) {
-            const float4 ai = sq.addi[i];
             tp.rad[0][g] = __fadd_rn(tp.rad[0][g], ad.x);
             tp.rad[1][g] = __fadd_rn(tp.rad[1][g], ad.y);
             tp.rad[2][g] = __fadd_rn(tp.rad[2][g], ad.z);
             if (b >= 1) {
+                const float4 ai = sq.addi[i];
                 tp.lind[0][g] = __fadd_rn(tp.lind[0][g], ai.x);
                 tp.lind[1][g] = __fadd_rn(tp.lind[1][g], ai.y);
                 tp.lind[2][g] = __fadd_rn(tp.lind[2][g], ai.z);
@@ -525,7 +553,6 @@ __global__ void __launch_bounds__(256) k_wreuse(const SceneDev* __restrict__ sce
             sq.o[ss] = make_float4(so.x, so.y, so.z, __int_as_float(tri));
             sq.d[ss] = make_float4(sd.x, sd.y, sd.z, __uint_as_float(sid));
             sq.add[ss] = make_float4(add.x, add.y, add.z, __int_as_float(vi));
-            sq.addi[ss] = make_float4(0.f, 0.f, 0.f, 0.f);
         }
     }
 }
@@ -568,7 +595,7 @@ __device__ __forceinline__ long long refill(RefillPool& rp, bool has, unsigned i
 }
 
 __global__ void __launch_bounds__(256, MR_CLOSEST_REFILL_MINB) k_wclosest_refill(const SceneDev* __restrict__ scenes,
-                                                         const ViewDev* __restrict__ views, QueueDev q,
+                                                         const ViewDev* __restrict__ views, int b, QueueDev q,
                                                          const unsigned int* count, QueueDev hq,
                                                          unsigned int* count_hit, unsigned int* fetch)
 {
@@ -605,7 +632,7 @@ __global__ void __launch_bounds__(256, MR_CLOSEST_REFILL_MINB) k_wclosest_refill
                 hq.o[slot] = make_float4(T.best.t, T.best.u, T.best.v, __int_as_float(T.best.tri));
                 hq.d[slot] = qd;
                 hq.b[slot] = qb;
-                hq.bi[slot] = q.bi[i];
+                if (b >= BI_FROM) hq.bi[slot] = q.bi[i];
             }
             if (done) has = false;
         }
@@ -648,11 +675,11 @@ __global__ void MR_TRACE_BOUNDS k_wshadow_refill(const SceneDev* __restrict__ sc
                 has = false;
                 const uint64_t g = views[__float_as_int(ad.w)].offset + __float_as_uint(dd.w);
                 if (T.best.tri < 0) {
-                    const float4 ai = sq.addi[i];
                     tp.rad[0][g] = __fadd_rn(tp.rad[0][g], ad.x);
                     tp.rad[1][g] = __fadd_rn(tp.rad[1][g], ad.y);
                     tp.rad[2][g] = __fadd_rn(tp.rad[2][g], ad.z);
                     if (b >= 1) {
+                        const float4 ai = sq.addi[i];
                         tp.lind[0][g] = __fadd_rn(tp.lind[0][g], ai.x);
                         tp.lind[1][g] = __fadd_rn(tp.lind[1][g], ai.y);
                         tp.lind[2][g] = __fadd_rn(tp.lind[2][g], ai.z);
@@ -885,9 +912,10 @@ void mr_wave_record(const SceneDev* scenes, const ViewDev* views, int n_views, u
         cudaMemsetAsync(qc, 0, sizeof(unsigned int) * (5 * max_bounces + 3), st);
         cur_b = -1;
         mark(3, true);
-        k_wraygen<<<grid_cap(n, blk_g, cap_g), blk_g, 0, st>>>(views, n_views, rng, first, n, qa, tape, total, nvx,
-                                                               res);
-        keep_seeded(st, k_wraygen, seeded);
+        if (raster) {
+            k_wraygen<<<grid_cap(n, blk_g, cap_g), blk_g, 0, st>>>(views, n_views, rng, first, n, qa);
+            keep_seeded(st, k_wraygen, seeded);
+        }
         mark(3, false);
         QueueDev cur = qa, nxt = qb;
         for (int b = 0; b < max_bounces; ++b) {
@@ -925,15 +953,23 @@ void mr_wave_record(const SceneDev* scenes, const ViewDev* views, int n_views, u
                 }
             }
             // primary rays stay coherent in the plain stage kernel; work is counted there too, ray by ray
-            if (b > 0 && !wide && !count)
-                k_wclosest_refill<<<grid_c, 256, smem, st>>>(scenes, views, cur, cnt_in, hq, qc + 3 * b, fetch + 2 * b);
-            else
-                (keys ? (count ? k_wclosest<true, true, false>
-                               : (wide ? k_wclosest<false, true, true> : k_wclosest<false, true, false>))
-                      : (count ? k_wclosest<true, false, false>
-                               : (wide ? k_wclosest<false, false, true> : k_wclosest<false, false, false>)))<<<
-                    grid_cap(n, blk_c, cap_c), blk_c, stack_c, st>>>(
-                    scenes, views, b, cur, cnt_in, n, hq, qc + 3 * b, tape, total, counters, keys);
+            if (b > 0 && !wide && !count) {
+                k_wclosest_refill<<<grid_c, 256, smem, st>>>(scenes, views, b, cur, cnt_in, hq, qc + 3 * b,
+                                                             fetch + 2 * b);
+            } else {
+                const auto k = b > 0 ? (count ? k_wclosest<true, false, false, false>
+                                              : k_wclosest<false, false, true, false>)
+                               : keys ? (count  ? k_wclosest<true, true, false, true>
+                                         : wide ? k_wclosest<false, true, true, true>
+                                                : k_wclosest<false, true, false, true>)
+                                      : (count  ? k_wclosest<true, false, false, true>
+                                         : wide ? k_wclosest<false, false, true, true>
+                                                : k_wclosest<false, false, false, true>);
+                k<<<grid_cap(n, blk_c, cap_c), blk_c, stack_c, st>>>(scenes, views, rng, n_views, b, cur, first, cnt_in, n,
+                                                                     hq, qc + 3 * b, tape, total, nvx, res, counters,
+                                                                     keys);
+                if (b == 0 && !keys) keep_seeded(st, k_wclosest<false, false, false, true>, seeded);
+            }
             mark(0, false);
             mark(1, true);
             const bool reuse_b = b == 0 && res.ytex != nullptr;
@@ -1002,5 +1038,5 @@ int mr_wave_stage_pairs(int n_waves, int max_bounces) { return n_waves * (1 + 3 
 int mr_wave_launches(int n_waves, int max_bounces, bool reuse, int temporal, int raster_launches, bool bin)
 {
     const int extra = (reuse ? 1 : 0) + (temporal == 2 ? 1 : 0) + (temporal ? 1 : 0) + (bin ? 3 * (max_bounces - 1) : 0);
-    return n_waves * (2 + 3 * max_bounces + extra) + 1 + raster_launches;
+    return n_waves * (1 + 3 * max_bounces + extra) + 1 + raster_launches;
 }
