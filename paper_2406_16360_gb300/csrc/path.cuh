@@ -123,11 +123,15 @@ __device__ __forceinline__ void tape_directions(const TapeDev& tp, uint64_t g, c
     tp.pind[g] = out.c_pind;
 }
 
-template <bool INTERP = true>
+// `thru(beta, bind)` gives the path's throughput and that of L_ind. It is asked once, after the
+// candidate loop, whose registers (64 at four blocks per SM, about 200 bytes spilled) the six values
+// would take: shade stage 1791 -> 1770 us on a ten-scene batch.
+template <bool INTERP = true, class Thru>
 __device__ __forceinline__ void shade_vertex(const SceneDev& s, int env_ok, const Rng& rng, uint32_t pixel,
                                              uint32_t smp, uint32_t view, int b, int B, int M, const Hit& h,
-                                             float3 d, float3 beta, float3 bind, VertexOut& out)
+                                             float3 d, const Thru& thru, VertexOut& out)
 {
+    float3 beta, bind;
     Shade sh;
     shade_at<INTERP>(s, h.tri, h.u, h.v, d, sh);
     const float3 wo = f3(-d.x, -d.y, -d.z);
@@ -221,6 +225,7 @@ __device__ __forceinline__ void shade_vertex(const SceneDev& s, int env_ok, cons
             const float gq = env_candidate(s, x.x, x.y, x.w, dir, tex);
             consider(j, x, dir, tex, gq, weigh(dir));
         }
+        thru(beta, bind);
         const float4 L = (sel >= 0) ? __ldg(s.env_texel + ytex) : make_float4(0.f, 0.f, 0.f, 0.f);
         const float phat_sel = lum(xyz(L)) * yfc_sel;
         out.wsum = wsum;
@@ -241,6 +246,8 @@ __device__ __forceinline__ void shade_vertex(const SceneDev& s, int env_ok, cons
             out.ytex = ytex;
             out.W = W;
         }
+    } else {
+        thru(beta, bind);
     }
     if (b < B - 1) {
         const uint4 x = rng.draw(pixel, smp, view, (uint32_t)b, PURPOSE_CONTINUE, 0u);

@@ -116,8 +116,12 @@ __global__ void __launch_bounds__(256, MR_SHADE_MINB) k_shade(SceneDev s, ViewDe
             h.u = hd.y;
             h.v = hd.z;
             h.tri = tri;
-            shade_vertex(s, env_ok, rng, pixel, smp, (uint32_t)v.index, b, v.bounces, M, h, d, xyz(hq.b[i]),
-                         xyz(hq.bi[i]), out);
+            shade_vertex(s, env_ok, rng, pixel, smp, (uint32_t)v.index, b, v.bounces, M, h, d,
+                         [&](float3& beta, float3& bind) {
+                             beta = xyz(hq.b[i]);
+                             bind = xyz(hq.bi[i]);
+                         },
+                         out);
             if (env_ok) n_cand += (unsigned long long)M;
             if (b == 0) {
                 tp.tri[g] = tri;
@@ -314,7 +318,12 @@ __device__ __forceinline__ void persistent_body(const SceneDev* __restrict__ sce
         if (has_hit) {
             const SceneDev& s = *sp;
             if (b == 0) tri0 = h.tri;
-            shade_vertex(s, env_ok, rng, pixel, smp, vidx, b, B, M, h, d, beta, bind, out);
+            shade_vertex(s, env_ok, rng, pixel, smp, vidx, b, B, M, h, d,
+                         [&](float3& be, float3& bi) {
+                             be = beta;
+                             bi = bind;
+                         },
+                         out);
             n_cand += (env_ok && M > 0) ? (unsigned long long)M : 0ull;
             if (b == 0) {
                 cand0 = out.cand;

@@ -284,8 +284,7 @@ __global__ void __launch_bounds__(256, MR_SHADE_MINB) k_wshade(const SceneDev* _
         if (i < n) {
             const float4 hd = hq.o[i];
             const float4 qd = hq.d[i];
-            const float4 qb = hq.b[i];
-            vi = __float_as_int(qb.w);
+            vi = __float_as_int(hq.b[i].w);
             const ViewDev& v = views[vi];
             const SceneDev& s = scenes[v.scene];
             sid = __float_as_uint(qd.w);
@@ -298,8 +297,12 @@ __global__ void __launch_bounds__(256, MR_SHADE_MINB) k_wshade(const SceneDev* _
             h.v = hd.z;
             h.tri = tri;
             const int env_ok = *s.env_ok_dev;
-            shade_vertex<INTERP>(s, env_ok, rng, pixel, smp, (uint32_t)v.index, b, v.bounces, M, h, xyz(qd), xyz(qb),
-                         b >= BI_FROM ? xyz(hq.bi[i]) : f3(1.f, 1.f, 1.f), out);
+            shade_vertex<INTERP>(s, env_ok, rng, pixel, smp, (uint32_t)v.index, b, v.bounces, M, h, xyz(qd),
+                                 [&](float3& beta, float3& bind) {
+                                     beta = xyz(hq.b[i]);
+                                     bind = b >= BI_FROM ? xyz(hq.bi[i]) : f3(1.f, 1.f, 1.f);
+                                 },
+                                 out);
             if (env_ok) n_cand += (unsigned long long)M;
             if (b == 0) {
                 tp.tri[g] = tri;
