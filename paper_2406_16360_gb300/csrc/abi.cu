@@ -504,6 +504,14 @@ static mirres_status stage_events(mirres_context* ctx, int pairs)
     return MIRRES_OK;
 }
 
+// A context whose wavefront shape nobody set runs its waves as two chains of half the size, so that a
+// wave's stages fill the SMs that the last long rays of the other's leave idle (a launch's longest ray
+// takes some 30 us whatever its size): 12 views of config 3 136.8 -> 131.6 ms, config-2 step 2634 ->
+// 2478 us, ten-scene batch 4565 -> 4380 us, FULL adjoint step 1772 -> 1751 us. A call of up to 2^25
+// samples is shared out evenly; below 2^17 samples the launches of a second chain cost what it gives
+// (64 x 64 preview: no difference). The queues hold what one chain's did. Renders that record stage
+// events keep one chain: with two, a stage's time holds the other's work.
+constexpr uint64_t kMinPairedWave = 1ull << 16;
 static mirres_status render_wave(mirres_context* ctx, const std::vector<SceneDev>& sdev,
                                  const std::vector<ViewDev>& vdev, uint64_t total, float* const* images, void* tape,
                                  int M, Rng rng, int flags, int nvx, int reuse_k, int reuse_radius, int temporal,
@@ -519,7 +527,14 @@ static mirres_status render_wave(mirres_context* ctx, const std::vector<SceneDev
         pixoff[(size_t)i] = total_pix;
         total_pix += (uint64_t)vdev[(size_t)i].width * vdev[(size_t)i].height;
     }
-    uint64_t kWave = 1ull << ctx->wave_shape.wave_log2;
+    mirres_wave_shape shape = ctx->wave_shape;
+    const bool paired = ctx->wave_default && !(flags & 1);
+    if (paired) {
+        shape.wave_log2 -= 1;
+        shape.branches = 2;
+    }
+    uint64_t kWave = 1ull << shape.wave_log2;
+    if (paired) kWave = std::min(kWave, std::max(((total + 1) / 2 + 255) / 256 * 256, kMinPairedWave));
     if (reuse) {
         // waves hold whole views (a pixel's neighbours must have been shaded in the same wave):
         // a view larger than the shape's wave gets a wave of its own size
@@ -543,7 +558,8 @@ static mirres_status render_wave(mirres_context* ctx, const std::vector<SceneDev
         for (uint64_t f = 0; f < total; f += wave) wave_first.push_back(f);
     }
     const int n_waves = (int)wave_first.size();
-    const int nb = std::min(ctx->wave_shape.branches, n_waves);  // chains of waves
+    int nb = std::min(shape.branches, n_waves);  // chains of waves
+    if (paired && nb > 1 && 2 * wave > 1ull << ctx->wave_shape.wave_log2) nb = 1;  // (reuse: a view beyond half a wave)
     Carver plan(nullptr);
     plan.take<char>(tape ? 0 : tape_bytes_per_sample(nvx) * total);
     plan.take<ViewDev>((size_t)n_views);
@@ -622,7 +638,7 @@ static mirres_status render_wave(mirres_context* ctx, const std::vector<SceneDev
     key.tape = tp;
     key.ws = ctx->ws.ptr;
     key.ws_bytes = ctx->ws.bytes;
-    key.shape = ctx->wave_shape;
+    key.shape = shape;
     static_assert(sizeof(GraphKey) <= sizeof(ctx->graph_key), "graph key too large");
     GraphKey have;
     std::memcpy(&have, ctx->graph_key, sizeof(have));
@@ -667,7 +683,7 @@ static mirres_status render_wave(mirres_context* ctx, const std::vector<SceneDev
                        ctx->sm_count, (flags & 1) ? ctx->stage_events : nullptr,
                        (flags & 1) ? ctx->stage_kind : nullptr, nvx, (flags & 2) != 0, reuse_k, reuse_radius, res,
                        temporal, temporal_cap, hist, vdev.data(), sdev.data(), (flags & 4) != 0, bin,
-                       ctx->wave_shape, &ctx->seeded);
+                       shape, &ctx->seeded);
         ctx->stage_pairs = (flags & 1) ? pairs : 0;
         cudaGraph_t g = nullptr;
         const cudaError_t ec = cudaStreamEndCapture(ctx->capture_stream, &g);
@@ -923,6 +939,7 @@ extern "C" mirres_status mirres_set_wave_shape(mirres_context* ctx, const mirres
     const mirres_wave_shape w = shape ? *shape : default_wave_shape();
     MR_TRY(check_wave_shape(w));
     ctx->wave_shape = w;
+    ctx->wave_default = shape == nullptr;
     return MIRRES_OK;
 }
 
@@ -995,6 +1012,8 @@ extern "C" mirres_status mirres_autotune_wave(mirres_context* ctx, mirres_scene*
     }
     const Rng rng = make_rng(params);
     const mirres_wave_shape keep = ctx->wave_shape;
+    const bool keep_default = ctx->wave_default;
+    ctx->wave_default = false;  // every candidate as it is given
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     mirres_status status = MIRRES_OK;
     // one render that captures the graph and warms caches and clocks, then `timed` renders of
@@ -1086,6 +1105,7 @@ extern "C" mirres_status mirres_autotune_wave(mirres_context* ctx, mirres_scene*
     cudaFree(img_buf);
     if (status != MIRRES_OK) {
         ctx->wave_shape = keep;
+        ctx->wave_default = keep_default;
         return status;
     }
     ctx->wave_shape = best;
