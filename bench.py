@@ -39,14 +39,14 @@ DEMOD_REPS = 5
 
 # DRAM bytes per unit of the three stage kernels (closest-hit ray, RIS candidate, shadow ray),
 # from one ncu capture (dram__bytes_read.sum + dram__bytes_write.sum) of the first render's
-# launches on config 3 reduced to 2 views, divided by that render's unit counts; the 1-view
-# capture gives per-unit figures within 2%, so traffic is taken to grow in proportion and is
+# launches on config 3 reduced to 2 views, divided by that render's unit counts; the per-unit
+# figures changed by 2% between 1 and 2 views, so traffic is taken to grow in proportion and is
 # scaled to the bench's launches by their unit counts. Valid only for the kernel sources they
 # were measured on (SHA-256 prefix of wave.cu, device.cuh, path.cuh, bvh.cu, env.cu); otherwise
 # null.
 TRAFFIC_SOURCES = ("wave.cu", "device.cuh", "path.cuh", "bvh.cu", "env.cu")
-TRAFFIC_SHA = "618e3614140c8c45"
-TRAFFIC_PER_UNIT = {"closest": 81.75, "shade": 12.09, "shadow": 125.11}
+TRAFFIC_SHA = "d988d2c01b8c23a9"
+TRAFFIC_PER_UNIT = {"closest": 53.66, "shade": 10.69, "shadow": 113.29}
 
 
 def _traffic_valid():
