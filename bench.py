@@ -45,7 +45,7 @@ DEMOD_REPS = 5
 # were measured on (SHA-256 prefix of wave.cu, device.cuh, path.cuh, bvh.cu, env.cu); otherwise
 # null.
 TRAFFIC_SOURCES = ("wave.cu", "device.cuh", "path.cuh", "bvh.cu", "env.cu")
-TRAFFIC_SHA = "d988d2c01b8c23a9"
+TRAFFIC_SHA = "f601da34acf72a93"
 TRAFFIC_PER_UNIT = {"closest": 53.66, "shade": 10.69, "shadow": 113.29}
 
 

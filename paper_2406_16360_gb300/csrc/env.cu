@@ -198,7 +198,7 @@ __device__ __forceinline__ int search_warp(const unsigned long long* __restrict_
 // n - 1. A block takes GUIDE_TILE consecutive buckets: two searches over the whole table find the
 // texels its first and last bucket fall on, the thresholds between them (about an eighth of the
 // buckets) go to shared memory and every bucket searches there: ~7 steps instead of 19 through
-// L2 at 1024 x 512 (54 us for the 4.2 M buckets before, now 36).
+// L2 at 1024 x 512 (54 us for the 4.2 M buckets before, now 38 with GUIDE_MORE).
 constexpr int GUIDE_TILE = 2048, GUIDE_SHARED = 1024;
 __global__ void __launch_bounds__(256) k_env_flat_guide(const unsigned long long* __restrict__ flat, int n, int g,
                                                         int shift, uint32_t* __restrict__ guide)
