@@ -944,7 +944,12 @@ __global__ void __launch_bounds__(256) k_tex_pack(const SceneDev* __restrict__ s
     }
 }
 
-// every scene's packed accumulators added to the caller's gradient arrays
+// Every scene's packed accumulators added to the caller's gradient arrays, atomically: scenes of one
+// call (all in flight together) may share an array, and so may calls on other streams.
+__device__ __forceinline__ void add_grad(float* p, size_t i, float x)
+{
+    if (p && x != 0.0f) atomicAdd(p + i, x);
+}
 __global__ void __launch_bounds__(256) k_grads_unpack(const SceneDev* __restrict__ scenes, const GradDev* __restrict__ grads)
 {
     const SceneDev& s = scenes[blockIdx.y];
@@ -953,26 +958,26 @@ __global__ void __launch_bounds__(256) k_grads_unpack(const SceneDev* __restrict
     const uint64_t n = (uint64_t)n_tex + n_env + n_verts;
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
         float* dst;
+        uint64_t k;
         float4 v;
         if (i < n_tex) {
-            v = __ldcs(g.ptex + 2 * i);
-            if (g.rough) g.rough[i] += v.w;
-            if (g.metal) g.metal[i] += __ldcs(g.ptex + 2 * i + 1).x;
-            dst = g.albedo ? g.albedo + 3 * i : nullptr;
+            k = i;
+            v = __ldcs(g.ptex + 2 * k);
+            add_grad(g.rough, k, v.w);
+            add_grad(g.metal, k, __ldcs(g.ptex + 2 * k + 1).x);
+            dst = g.albedo;
         } else if (i < (uint64_t)n_tex + n_env) {
-            const uint64_t k = i - n_tex;
+            k = i - n_tex;
             v = __ldcs(g.penv + k);
-            dst = g.env ? g.env + 3 * k : nullptr;
+            dst = g.env;
         } else {
-            const uint64_t k = i - n_tex - n_env;
+            k = i - n_tex - n_env;
             v = __ldcs(g.pvert + k);
-            dst = g.verts ? g.verts + 3 * k : nullptr;
+            dst = g.verts;
         }
-        if (dst) {
-            dst[0] += v.x;
-            dst[1] += v.y;
-            dst[2] += v.z;
-        }
+        add_grad(dst, 3 * k, v.x);
+        add_grad(dst, 3 * k + 1, v.y);
+        add_grad(dst, 3 * k + 2, v.z);
     }
 }
 
