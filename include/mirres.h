@@ -406,7 +406,8 @@ mirres_status mirres_render_noalloc(mirres_scene* const* scenes, int32_t n_scene
  * visibility, every sampling decision, p_ind and L_ind held fixed) are scattered into the
  * texels of albedo / roughness / metallic (bilinear weights), the env texel of the selected
  * candidate and of escaping primary rays, and the three vertices of the primary triangle
- * (through the intersection barycentrics and the face normal). Warp-aggregated FP32 atomics.
+ * (through the intersection barycentrics and the face normal). Warp-aggregated FP32 atomics, so that
+ * several scenes of a call, and calls on other streams, may name the same destination.
  *   d_images[v]  device [height][width][3] = dL/dI (e.g. 2 (I - I_ref) for Eq. loss_pbr)
  *   grads[s]     gradient destinations of scene s (host array of n_scenes structs)
  * The views, params and scenes must be those of the render that wrote `tape`. */
