@@ -1189,16 +1189,24 @@ static mirres_status backward_impl(mirres_context* ctx, mirres_scene* const* sce
     // save 15 to 30 ps a sample. One view, us a call, direct / packed: 512 x 512 textures 43 / 54 at
     // 2^18 samples, 66 / 75 at 2^19, 230 / 215 at 2^21; 1000 x 1000 and 131k env texels 68 / 113 at
     // 2^19, 239 / 228 at 2^21. The line lies between: 2^20 samples, and one per parameter.
-    uint64_t n_tex = 0, n_vec = 0, most_tex = 0, most = 0;
+    // Accumulators are kept for the destinations that are asked for only.
+    struct AccCounts {
+        size_t tex, env, verts;  // records: two float4 a texel, one an env texel or a vertex
+    };
+    std::vector<AccCounts> want((size_t)n_scenes);
+    uint64_t n_tex = 0, n_vec = 0, n_acc = 0, most_tex = 0, most = 0;
     for (int i = 0; i < n_scenes; ++i) {
         const mirres_scene_desc& d = scenes[i]->desc;
-        gdev[(size_t)i] = GradDev{grads[i].albedo, grads[i].roughness, grads[i].metallic, grads[i].env, grads[i].verts,
-                                  nullptr, nullptr, nullptr};
-        const uint64_t nt = (uint64_t)d.tex_w * d.tex_h, nv = (uint64_t)d.env_w * d.env_h + (uint64_t)d.n_verts;
+        const mirres_grads& g = grads[i];
+        gdev[(size_t)i] = GradDev{g.albedo, g.roughness, g.metallic, g.env, g.verts, nullptr, nullptr, nullptr};
+        const uint64_t nt = (uint64_t)d.tex_w * d.tex_h, ne = (uint64_t)d.env_w * d.env_h, nv = (uint64_t)d.n_verts;
+        AccCounts& w = want[(size_t)i];
+        w = AccCounts{(g.albedo || g.roughness || g.metallic) ? nt : 0, g.env ? ne : 0, g.verts ? nv : 0};
         n_tex += nt;
-        n_vec += nv;
+        n_vec += ne + nv;
+        n_acc += 2 * w.tex + w.env + w.verts;
         most_tex = std::max(most_tex, nt);
-        most = std::max(most, nt + nv);
+        most = std::max<uint64_t>(most, w.tex + w.env + w.verts);
     }
     bool packed = total >= MR_PACK_MIN && total >= MR_PACK_RATIO * (n_tex + n_vec) && most_tex < (1u << 29) &&
                   n_scenes <= 65535;
@@ -1210,7 +1218,7 @@ static mirres_status backward_impl(mirres_context* ctx, mirres_scene* const* sce
         plan.take<GradDev>((size_t)n_scenes);
         plan.take<char>(nvx > 0 ? mr_full_scratch_bytes() : 0);
         plan.take<float4>(with_packed ? 2 * n_tex : 0);
-        plan.take<float4>(with_packed ? 2 * n_tex + n_vec : 0);
+        plan.take<float4>(with_packed ? n_acc : 0);
         return plan.off;
     };
     if (packed && ws_reserve(ctx, plan_bytes(true)) != MIRRES_OK) packed = false;  // no room: without them
@@ -1222,18 +1230,19 @@ static mirres_status backward_impl(mirres_context* ctx, mirres_scene* const* sce
     GradDev* d_grads = cv.take<GradDev>((size_t)n_scenes);
     void* full_scratch = cv.take<char>(nvx > 0 ? mr_full_scratch_bytes() : 0);
     float4* tex8 = cv.take<float4>(packed ? 2 * n_tex : 0);
-    float4* acc = cv.take<float4>(packed ? 2 * n_tex + n_vec : 0);
+    float4* acc = cv.take<float4>(packed ? n_acc : 0);
     if (packed) {
-        MR_CUDA(cudaMemsetAsync(acc, 0, sizeof(float4) * (2 * n_tex + n_vec), st));
+        if (n_acc) MR_CUDA(cudaMemsetAsync(acc, 0, sizeof(float4) * n_acc, st));
         for (int i = 0; i < n_scenes; ++i) {
             const mirres_scene_desc& d = scenes[i]->desc;
-            const size_t nt = (size_t)d.tex_w * d.tex_h, ne = (size_t)d.env_w * d.env_h;
+            const AccCounts& w = want[(size_t)i];
+            GradDev& g = gdev[(size_t)i];
             sdev[(size_t)i].tex8 = tex8;
-            gdev[(size_t)i].ptex = acc;
-            gdev[(size_t)i].penv = acc + 2 * nt;
-            gdev[(size_t)i].pvert = acc + 2 * nt + ne;
-            tex8 += 2 * nt;
-            acc += 2 * nt + ne + (size_t)d.n_verts;
+            tex8 += 2 * (size_t)d.tex_w * d.tex_h;
+            g.ptex = w.tex ? acc : nullptr;
+            g.penv = w.env ? acc + 2 * w.tex : nullptr;
+            g.pvert = w.verts ? acc + 2 * w.tex + w.env : nullptr;
+            acc += 2 * w.tex + w.env + w.verts;
         }
     }
     MR_CUDA(cudaMemcpyAsync(d_views, vdev.data(), sizeof(ViewDev) * vdev.size(), cudaMemcpyHostToDevice, st));
@@ -1253,7 +1262,7 @@ static mirres_status backward_impl(mirres_context* ctx, mirres_scene* const* sce
     else
         mr_launch_backward(d_scenes, d_views, n_views, total, make_rng(params), d_dimg, d_grads, tape, ctx->counters,
                            ctx->sm_count, st, nvx, full_scratch, interp, packed);
-    if (packed) mr_launch_grads_unpack(d_scenes, d_grads, n_scenes, most, ctx->sm_count, st);
+    if (packed && most) mr_launch_grads_unpack(d_scenes, d_grads, n_scenes, most, ctx->sm_count, st);
     // interpolated normals: d loss / d vertex normal to the vertices of the incident faces
     for (int i = 0; i < n_scenes; ++i)
         if (scenes[i]->normals && grads[i].verts && scenes[i]->gvn) {
@@ -1262,7 +1271,7 @@ static mirres_status backward_impl(mirres_context* ctx, mirres_scene* const* sce
         }
     MR_CUDA(cudaGetLastError());
     const uint64_t full_chunk = mr_full_chunk();
-    ctx->host_launches += 1 + (unsigned long long)normals_passes + (packed ? 2ull : 0ull) +
+    ctx->host_launches += 1 + (unsigned long long)normals_passes + (packed ? (most ? 2ull : 1ull) : 0ull) +
                           (nvx > 0 ? 4 * ((total + full_chunk - 1) / full_chunk) : 0);
     return MIRRES_OK;
 }

@@ -887,45 +887,52 @@ __global__ void __launch_bounds__(256, MR_BWD_MINB) k_backward(const SceneDev* _
                 // samples, mostly background under a 32 x 16 env, 5.52 ms, so 0.42; a sun of 99% of the energy
                 // 0.90 -> 0.72 ms; the chain in every warp with a pair 0.74 ms, and 1.67 instead of 1.62 ms on two
                 // views of config 3.)
-                const int ek = mine ? env_key : -1;
-                const unsigned same = __match_any_sync(MR_FULL, ek);
-                auto emit_env = [&](int t, const float (&x)[3]) { red4(gd.penv + t, x[0], x[1], x[2], 0.0f); };
-                if (__any_sync(MR_FULL, ek >= 0 && __popc(same) > 2)) {
-                    scatter_agg<3>(ek, env_v, emit_env);
-                } else {
-                    const unsigned other = same & ~(1u << lane_id());
-                    const int from = other ? __ffs(other) - 1 : lane_id();
-                    float x[3];
+                if (gd.penv) {
+                    const int ek = mine ? env_key : -1;
+                    const unsigned same = __match_any_sync(MR_FULL, ek);
+                    auto emit_env = [&](int t, const float (&x)[3]) { red4(gd.penv + t, x[0], x[1], x[2], 0.0f); };
+                    if (__any_sync(MR_FULL, ek >= 0 && __popc(same) > 2)) {
+                        scatter_agg<3>(ek, env_v, emit_env);
+                    } else {
+                        const unsigned other = same & ~(1u << lane_id());
+                        const int from = other ? __ffs(other) - 1 : lane_id();
+                        float x[3];
 #pragma unroll
-                    for (int c = 0; c < 3; ++c) {
-                        const float o = __shfl_sync(MR_FULL, env_v[c], from);
-                        x[c] = env_v[c] + (other ? o : 0.0f);
+                        for (int c = 0; c < 3; ++c) {
+                            const float o = __shfl_sync(MR_FULL, env_v[c], from);
+                            x[c] = env_v[c] + (other ? o : 0.0f);
+                        }
+                        if (ek >= 0 && from >= lane_id()) emit_env(ek, x);
                     }
-                    if (ek >= 0 && from >= lane_id()) emit_env(ek, x);
                 }
                 // taps by footprint (its first texel and whether it is clamped in x and y), corners by
                 // triangle: one match and one chain of shuffles for all their sums
-                const int foot = (mine && tex_key[0] >= 0) ? (tex_key[0] << 2) + (tex_key[1] != tex_key[0]) +
-                                                                 2 * (tex_key[2] != tex_key[0])
-                                                           : -1;
-                float tv[20], cv[9];
+                if (gd.ptex) {
+                    const int foot = (mine && tex_key[0] >= 0) ? (tex_key[0] << 2) + (tex_key[1] != tex_key[0]) +
+                                                                     2 * (tex_key[2] != tex_key[0])
+                                                               : -1;
+                    float tv[20];
 #pragma unroll
-                for (int q = 0; q < 20; ++q) tv[q] = tex_v[q / 5][q % 5];
+                    for (int q = 0; q < 20; ++q) tv[q] = tex_v[q / 5][q % 5];
+                    scatter_agg<20>(foot, tv, [&](int, const float (&x)[20]) {
 #pragma unroll
-                for (int q = 0; q < 9; ++q) cv[q] = vert_v[q / 3][q % 3];
-                scatter_agg<20>(foot, tv, [&](int, const float (&x)[20]) {
+                        for (int q = 0; q < 4; ++q) {
+                            float4* const t = gd.ptex + 2 * (size_t)tex_key[q];
+                            red4(t, x[5 * q], x[5 * q + 1], x[5 * q + 2], x[5 * q + 3]);
+                            if (gd.metal) atomicAdd(&t[1].x, x[5 * q + 4]);
+                        }
+                    });
+                }
+                if (gd.pvert) {
+                    float cv[9];
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        float4* const t = gd.ptex + 2 * (size_t)tex_key[q];
-                        red4(t, x[5 * q], x[5 * q + 1], x[5 * q + 2], x[5 * q + 3]);
-                        atomicAdd(&t[1].x, x[5 * q + 4]);
-                    }
-                });
-                scatter_agg<9>(mine ? tri_key : -1, cv, [&](int, const float (&x)[9]) {
+                    for (int q = 0; q < 9; ++q) cv[q] = vert_v[q / 3][q % 3];
+                    scatter_agg<9>(mine ? tri_key : -1, cv, [&](int, const float (&x)[9]) {
 #pragma unroll
-                    for (int c = 0; c < 3; ++c)
-                        if (vert_key[c] >= 0) red4(gd.pvert + vert_key[c], x[3 * c], x[3 * c + 1], x[3 * c + 2], 0.0f);
-                });
+                        for (int c = 0; c < 3; ++c)
+                            if (vert_key[c] >= 0) red4(gd.pvert + vert_key[c], x[3 * c], x[3 * c + 1], x[3 * c + 2], 0.0f);
+                    });
+                }
             } else {
                 scatter_agg<3>(mine ? env_key : -1, env_v, EmitEnv{gd.env});
 #pragma unroll
@@ -974,8 +981,8 @@ __global__ void __launch_bounds__(256) k_grads_unpack(const SceneDev* __restrict
 {
     const SceneDev& s = scenes[blockIdx.y];
     const GradDev g = grads[blockIdx.y];
-    const uint32_t n_tex = (uint32_t)s.tw * (uint32_t)s.th, n_env = (uint32_t)s.ew * (uint32_t)s.eh, n_verts = (uint32_t)s.n_verts;
-    const uint64_t n = (uint64_t)n_tex + n_env + n_verts;
+    const uint32_t n_tex = g.ptex ? (uint32_t)s.tw * (uint32_t)s.th : 0u, n_env = g.penv ? (uint32_t)s.ew * (uint32_t)s.eh : 0u;
+    const uint64_t n = (uint64_t)n_tex + n_env + (g.pvert ? (uint32_t)s.n_verts : 0u);
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
         float* dst;
         uint64_t k;
@@ -984,7 +991,7 @@ __global__ void __launch_bounds__(256) k_grads_unpack(const SceneDev* __restrict
             k = i;
             v = __ldcs(g.ptex + 2 * k);
             add_grad(g.rough, k, v.w);
-            add_grad(g.metal, k, __ldcs(g.ptex + 2 * k + 1).x);
+            if (g.metal) add_grad(g.metal, k, __ldcs(g.ptex + 2 * k + 1).x);
             dst = g.albedo;
         } else if (i < (uint64_t)n_tex + n_env) {
             k = i - n_tex;

@@ -50,7 +50,8 @@ struct GradDev {
     float* metal;
     float* env;
     float* verts;
-    // packed accumulators of one call (null: none), added to the above by mr_launch_grads_unpack:
+    // packed accumulators of one call (null: none, or none of their destinations is asked for), added to
+    // the above by mr_launch_grads_unpack:
     // per texel (albedo, roughness) (metallic, -), per env texel and per vertex (x, y, z, -)
     float4* ptex;
     float4* penv;
