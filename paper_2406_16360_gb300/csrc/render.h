@@ -121,7 +121,8 @@ void mr_launch_eawt_pack_adjoint(const float* d, const float* ik, float4* out, i
 // level lstep (taps 2^lstep pixels apart); g: 32-byte G-buffer records
 void mr_launch_eawt_level(const float4* c, const float4* g, int N, int W, int H, int lstep, float inv_rt2, float inv_n2,
                           float inv_x2, float4* cout, float* out3, float* ikout, cudaStream_t st);
-// gin: the gradient over the level's k; ik_next: 1 / k of the level below, null at the first
+// gin: the gradient and 1 / k of the level; ik_next: 1 / k of the level below (null at the first, which
+// writes out3)
 void mr_launch_eawt_level_adjoint(const float4* gin, const float4* c, const float4* g, int N, int W, int H, int lstep,
                                   float inv_rt2, float inv_n2, float inv_x2, float4* gout, float* out3,
                                   const float* ik_next, cudaStream_t st);
