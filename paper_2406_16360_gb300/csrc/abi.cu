@@ -47,7 +47,7 @@ static const size_t kQueueCnt = 1024;
 SceneDev mr_scene_dev(const mirres_scene* s)
 {
     SceneDev d;
-    d.nodes = MR_DFS_NODES ? s->dnodes : s->nodes;
+    d.nodes = s->dnodes;
     d.ptri = s->ptri;
     d.leaf_of = s->leaf_of;
     d.tris = s->desc.tris;

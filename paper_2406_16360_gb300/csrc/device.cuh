@@ -28,9 +28,6 @@
 #else
 #define MR_TRACE_BOUNDS __launch_bounds__(256)
 #endif
-#ifndef MR_DFS_NODES
-#define MR_DFS_NODES 1  // traversal nodes in depth-first preorder (else the builders' order)
-#endif
 #ifndef MR_NODE_LD256
 #define MR_NODE_LD256 1  // traversal nodes read with two 256-bit loads (2.5% faster traversal stages)
 #endif
