@@ -70,7 +70,8 @@
 #define MR_SSTACK 16
 #endif
 #define MR_LSTACK (64 - MR_SSTACK)
-static_assert(MR_REFILL_STEPS % 2 == 0, "leaves are tested after every second visit");
+static_assert(MR_REFILL_STEPS >= 2 && MR_REFILL_STEPS % 2 == 0, "leaves are tested after every second visit");
+static_assert(MR_PEND >= 2, "a visit may put two leaves aside");
 static_assert(MR_SSTACK >= 8 && MR_SSTACK <= 56, "MR_SSTACK out of range");
 // the wide traversal's stack of 8-byte node groups: the first MR_SSTACK / 2 in the same shared
 // memory column, the rest local; a wide tree is at most as deep as its binary tree (<= 63)
