@@ -89,6 +89,7 @@ SceneDev mr_scene_dev(const mirres_scene* s)
 static mirres_status ws_reserve(mirres_context* ctx, size_t bytes)
 {
     if (bytes <= ctx->ws.bytes) return MIRRES_OK;
+    ctx->ws_refused = 0;
     if (ctx->ws.ptr) {
         MR_CUDA(cudaDeviceSynchronize());
         cudaFree(ctx->ws.ptr);
@@ -111,6 +112,28 @@ static mirres_status ws_reserve(mirres_context* ctx, size_t bytes)
     }
     ctx->ws.bytes = want;
     return MIRRES_OK;
+}
+
+// Grows the workspace for scratch that the call can do without: where there is no room the old one stays
+// (the forward's captured graph and its queues live in it), and the size is not tried again until the
+// workspace has been laid out anew.
+static bool ws_try(mirres_context* ctx, size_t bytes)
+{
+    if (bytes <= ctx->ws.bytes) return true;
+    if (ctx->ws_refused && bytes >= ctx->ws_refused) return false;
+    void* p = nullptr;
+    if (cudaMalloc(&p, bytes) != cudaSuccess) {
+        cudaGetLastError();
+        ctx->ws_refused = bytes;
+        return false;
+    }
+    if (ctx->ws.ptr) {
+        cudaDeviceSynchronize();
+        cudaFree(ctx->ws.ptr);
+    }
+    ctx->ws.ptr = p;
+    ctx->ws.bytes = bytes;
+    return true;
 }
 
 struct Carver {
@@ -1221,7 +1244,7 @@ static mirres_status backward_impl(mirres_context* ctx, mirres_scene* const* sce
         plan.take<float4>(with_packed ? n_acc : 0);
         return plan.off;
     };
-    if (packed && ws_reserve(ctx, plan_bytes(true)) != MIRRES_OK) packed = false;  // no room: without them
+    if (packed) packed = ws_try(ctx, plan_bytes(true));  // no room: without them
     if (!packed) MR_TRY(ws_reserve(ctx, plan_bytes(false)));
     Carver cv(ctx->ws.ptr);
     ViewDev* d_views = cv.take<ViewDev>((size_t)n_views);

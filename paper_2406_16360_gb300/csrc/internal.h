@@ -43,6 +43,7 @@ struct mirres_context {
     int device = 0;
     int sm_count = 0;
     Workspace ws;
+    size_t ws_refused = 0;  // bytes that there was no room for (ws_try); 0: none tried since ws was laid out
     unsigned long long* counters = nullptr;  // device [CNT_N]
     unsigned int* queue_cnt = nullptr;       // device scratch counters [64]
     cudaStream_t last_stream = nullptr;
