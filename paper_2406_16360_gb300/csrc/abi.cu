@@ -531,10 +531,10 @@ static mirres_status stage_events(mirres_context* ctx, int pairs)
 // wave's stages fill the SMs that the last long rays of the other's leave idle (a launch's longest ray
 // takes some 30 us whatever its size): 12 views of config 3 136.8 -> 131.6 ms, config-2 step 2634 ->
 // 2478 us, ten-scene batch 4565 -> 4380 us, FULL adjoint step 1772 -> 1751 us. A call of up to 2^25
-// samples is shared out evenly; below 2^17 samples the launches of a second chain cost what it gives
-// (64 x 64 preview: no difference). The queues hold what one chain's did. Renders that record stage
-// events keep one chain: with two, a stage's time holds the other's work.
-constexpr uint64_t kMinPairedWave = 1ull << 16;
+// samples is shared out evenly. One below 2^17 samples keeps one chain: the launches of a second cost
+// what it gives (181 x 181 at 3 samples: 640 us either way). The queues hold what one chain's did.
+// Renders that record stage events keep one chain: with two, a stage's time holds the other's work.
+constexpr uint64_t kMinPaired = 1ull << 17;
 static mirres_status render_wave(mirres_context* ctx, const std::vector<SceneDev>& sdev,
                                  const std::vector<ViewDev>& vdev, uint64_t total, float* const* images, void* tape,
                                  int M, Rng rng, int flags, int nvx, int reuse_k, int reuse_radius, int temporal,
@@ -551,13 +551,13 @@ static mirres_status render_wave(mirres_context* ctx, const std::vector<SceneDev
         total_pix += (uint64_t)vdev[(size_t)i].width * vdev[(size_t)i].height;
     }
     mirres_wave_shape shape = ctx->wave_shape;
-    const bool paired = ctx->wave_default && !(flags & 1);
+    const bool paired = ctx->wave_default && !(flags & 1) && total >= kMinPaired;
     if (paired) {
         shape.wave_log2 -= 1;
         shape.branches = 2;
     }
     uint64_t kWave = 1ull << shape.wave_log2;
-    if (paired) kWave = std::min(kWave, std::max(((total + 1) / 2 + 255) / 256 * 256, kMinPairedWave));
+    if (paired) kWave = std::min(kWave, ((total + 1) / 2 + 255) / 256 * 256);
     if (reuse) {
         // waves hold whole views (a pixel's neighbours must have been shaded in the same wave):
         // a view larger than the shape's wave gets a wave of its own size

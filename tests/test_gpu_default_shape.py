@@ -1,0 +1,57 @@
+"""The default wavefront shape, two chains of half a wave, against one chain (the default's sizes with
+another grid for the shading kernel, which changes nothing but time): calls too small for two chains
+launch what one chain does, calls of several waves a chain and reuse views beyond half a wave give the
+same tape, images and history."""
+import pytest
+import torch
+
+from paper_2406_16360_gb300 import synth
+from tests.test_gpu_parity import M  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+ONE_CHAIN = dict(wave_log2=25, block=[256] * 4, blocks_per_sm=[8, 7, 8, 8], branches=1)
+
+
+def _render(M, sizes, shape, reuse=0, seeds=(3,)):  # noqa: F811
+    from paper_2406_16360_gb300.renderer import GpuWorkload
+    views = []
+    for k, (w, h, spp, bounces) in enumerate(sizes):
+        K, c2w = synth.look_at((0.3 * k, 1.5, 4.0), (0.0, 1.0, 0.0), w, h, 40.0)
+        views.append(synth.View(K, c2w, w, h, spp, bounces, 0))
+    ctx = M.mirres_context_create(0)
+    if shape is not None:
+        M.mirres_set_wave_shape(ctx, shape)
+    gw = GpuWorkload(synth.Workload("shape", [synth.tiny_scene(subdiv=1)], views, ris_m=2), 0, ctx=ctx)
+    tape, hist = torch.zeros_like(gw.new_tape()), gw.new_history() if reuse else None
+    kw = dict(reuse=(reuse, 8), temporal=2, history=hist) if reuse else {}
+    M.mirres_reset_counters(ctx)
+    for seed in seeds:
+        images, _ = gw.render(launch=1, tape=tape, seed=seed, **kw)
+    torch.cuda.synchronize()
+    counters = M.mirres_get_counters(ctx)
+    gw.close()
+    return [tape] + images + ([hist] if reuse else []), counters
+
+
+@pytest.mark.parametrize("samples", [65536, 65537, 131071, 131072])
+def test_two_chains_from_two_to_the_seventeen(M, samples):  # noqa: F811
+    a, ca = _render(M, [(samples, 1, 1, 2)], None)
+    b, cb = _render(M, [(samples, 1, 1, 2)], ONE_CHAIN)
+    assert all(torch.equal(x, y) for x, y in zip(a, b))
+    assert ca[:5] == cb[:5]
+    assert (ca[6] == cb[6]) == (samples < 1 << 17)  # kernel launches
+
+
+@pytest.mark.parametrize("sizes,reuse", [
+    ([(1, 1, 1, 1)], 0), ([(256, 257, 1, 2)], 0), ([(401, 127, 3, 1), (64, 33, 5, 2)], 0), ([(300, 200, 2, 1)] * 3, 4),
+    ([(512, 300, 2, 2), (31, 17, 3, 3)], 4),
+    ([(2048, 2048, 8, 2), (257, 1, 1, 1)], 0),  # 2^25 and 257 samples: three waves over two chains
+    ([(2900, 2900, 3, 2), (1024, 1000, 17, 1), (1111, 1000, 11, 2)], 0),
+    ([(2900, 2900, 2, 2), (300, 200, 2, 1)], 4),  # a reuse view beyond half a wave: one chain
+    ([(1024, 1024, 12, 2), (1000, 1024, 12, 1), (1024, 1001, 12, 2)], 4)])  # three waves of whole views
+def test_default_equals_one_chain(M, sizes, reuse):  # noqa: F811
+    seeds = (3, 4) if reuse else (3,)
+    a, ca = _render(M, sizes, None, reuse, seeds)
+    b, cb = _render(M, sizes, ONE_CHAIN, reuse, seeds)
+    assert all(torch.equal(x, y) for x, y in zip(a, b))
+    assert ca[:5] == cb[:5]
