@@ -320,9 +320,9 @@ mirres_status mirres_set_launch(mirres_context* ctx, int32_t block, int32_t bloc
  * The lane-refilling kernels that trace continuation rays (bounces >= 1) and shadow rays run
  * 256 threads in one resident wave of blocks whatever the shape; the shape sets the primary
  * rays' closest-hit kernel, shading and ray generation (and shadow rays on 8-wide BVHs).
- * Default: 2^25 samples, 256 threads and 8 blocks per SM for every stage, one chain; while it is not
- * set, renders without flags bit 0 (stage events) run a wave as two chains of half its size, with
- * the same ray queues in all. */
+ * Default: 2^25 samples, 256 threads and 8 blocks per SM for every stage, one chain. With these values
+ * (never set, restored, or read and set again) renders of 2^17 samples and more without flags bit 0
+ * (stage events) run a wave as two chains of half its size, with the same ray queues in all. */
 typedef struct {
     int32_t wave_log2;        /* samples per wave = 2^wave_log2, in [16, 28] */
     int32_t block[4];         /* 64, 128 or 256 */

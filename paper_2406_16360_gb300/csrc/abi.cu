@@ -459,6 +459,13 @@ static bool any_wide(const std::vector<SceneDev>& sdev)
 
 static mirres_wave_shape default_wave_shape() { return mirres_wave_shape{25, {256, 256, 256, 256}, {8, 8, 8, 8}, 1}; }
 
+static bool is_default(const mirres_wave_shape& w)
+{
+    const mirres_wave_shape d = default_wave_shape();
+    static_assert(sizeof(d) == 10 * sizeof(int32_t), "compared as plain words");
+    return std::memcmp(&w, &d, sizeof(d)) == 0;
+}
+
 static mirres_status check_wave_shape(const mirres_wave_shape& w)
 {
     if (w.wave_log2 < 16 || w.wave_log2 > 28) return arg_error("wave_log2 must be in [16, 28]");
@@ -527,7 +534,7 @@ static mirres_status stage_events(mirres_context* ctx, int pairs)
     return MIRRES_OK;
 }
 
-// A context whose wavefront shape nobody set runs its waves as two chains of half the size, so that a
+// A context with the default wavefront shape runs its waves as two chains of half the size, so that a
 // wave's stages fill the SMs that the last long rays of the other's leave idle (a launch's longest ray
 // takes some 30 us whatever its size): 12 views of config 3 136.8 -> 131.6 ms, config-2 step 2634 ->
 // 2478 us, ten-scene batch 4565 -> 4380 us, FULL adjoint step 1772 -> 1751 us. A call of up to 2^25
@@ -962,7 +969,7 @@ extern "C" mirres_status mirres_set_wave_shape(mirres_context* ctx, const mirres
     const mirres_wave_shape w = shape ? *shape : default_wave_shape();
     MR_TRY(check_wave_shape(w));
     ctx->wave_shape = w;
-    ctx->wave_default = shape == nullptr;
+    ctx->wave_default = is_default(w);  // also when read and set again
     return MIRRES_OK;
 }
 

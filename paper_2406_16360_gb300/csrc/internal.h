@@ -57,7 +57,7 @@ struct mirres_context {
     SeededNodes seeded;
     unsigned char graph_key[192] = {};
     mirres_wave_shape wave_shape = {25, {256, 256, 256, 256}, {8, 8, 8, 8}, 1};  // batched wavefront launch shape
-    bool wave_default = true;  // nobody set it: run as two chains of half the wave (render_wave)
+    bool wave_default = true;  // it is the default: run as two chains of half the wave (render_wave)
     cudaStream_t branch_stream[4] = {};  // [1..3]: the streams of wave chains 1..3 during capture
     cudaEvent_t branch_event[4] = {};    // [0]: fork, [1..3]: join of chains 1..3
     unsigned long long graph_launches = 0;  // kernel launches inside the graph

@@ -55,3 +55,15 @@ def test_default_equals_one_chain(M, sizes, reuse):  # noqa: F811
     b, cb = _render(M, sizes, ONE_CHAIN, reuse, seeds)
     assert all(torch.equal(x, y) for x, y in zip(a, b))
     assert ca[:5] == cb[:5]
+
+
+def test_default_read_and_set_again_stays_the_default(M):  # noqa: F811
+    sizes = [(512, 300, 2, 2)]
+    c = M.mirres_context_create(0)
+    shape = M.mirres_get_wave_shape(c)
+    c.close()
+    a, ca = _render(M, sizes, None)
+    b, cb = _render(M, sizes, shape)
+    one, c1 = _render(M, sizes, ONE_CHAIN)
+    assert all(torch.equal(x, y) and torch.equal(x, z) for x, y, z in zip(a, b, one))
+    assert ca[6] == cb[6] > c1[6]  # kernel launches: two waves, two waves, one
