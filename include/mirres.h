@@ -346,7 +346,8 @@ mirres_status mirres_get_wave_shape(mirres_context* ctx, mirres_wave_shape* out)
  * then two and three chains of waves (branches = 2, 3) at the chosen wave size and at half of
  * it, where the tuned views fill as many waves as chains, kept if faster still. Each shape is
  * rendered once to capture its graph, then timed (the fastest of two renders for the wave sizes
- * and chains).
+ * and chains). Last, from 2^17 samples, the shape found is timed against the default as it runs (two
+ * chains that share the batch evenly), without stage events, and the faster of the two is kept.
  * The result becomes the context's shape (mirres_set_wave_shape) and is written to *out, the
  * tuned forward's time to *out_ms. The tape must hold these views (it is overwritten); the
  * renders write temporary images (allocated and freed here). params as for mirres_render
