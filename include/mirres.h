@@ -315,11 +315,13 @@ mirres_status mirres_set_launch(mirres_context* ctx, int32_t block, int32_t bloc
 
 /* Launch shape of the batched wavefront (launch = 1; no counterpart in the paper): the wave size
  * -- samples per wave, which is the capacity of every ray queue -- and, per stage kernel
- * (index = stage: 0 closest hit, 1 shade + RIS (and the reuse kernels), 2 shadow rays, 3 ray
- * generation), the threads per block and the grid of its grid-stride loop in blocks per SM.
+ * (index = stage: 0 closest hit, which makes the camera rays it traces, 1 shade + RIS (and the reuse
+ * kernels), 2 shadow rays, 3 ray generation for the rasteriser, flags bit 2, the only one that reads
+ * camera rays from a queue), the threads per block and the grid of its grid-stride loop in blocks per SM.
  * The lane-refilling kernels that trace continuation rays (bounces >= 1) and shadow rays run
  * 256 threads in one resident wave of blocks whatever the shape; the shape sets the primary
- * rays' closest-hit kernel, shading and ray generation (and shadow rays on 8-wide BVHs).
+ * rays' closest-hit kernel, shading and the rasteriser's ray generation (and shadow rays on 8-wide
+ * BVHs).
  * Default: 2^25 samples, 256 threads and 8 blocks per SM for every stage, one chain. With these values
  * (never set, restored, or read and set again) renders of 2^17 samples and more without flags bit 0
  * (stage events) run a wave as two chains of half its size, with the same ray queues in all. */
@@ -341,7 +343,8 @@ mirres_status mirres_get_wave_shape(mirres_context* ctx, mirres_wave_shape* out)
 /* Autotuner of the batched wavefront: renders the first views of the batch (up to
  * budget_samples samples, at least one view; 0 = all) with the wavefront and CUDA events around
  * every stage, for each of a set of (threads per block, blocks per SM) pairs applied to all
- * stages at once; keeps the fastest pair per stage, then times the wave sizes 2^23, 2^24 and
+ * stages at once; keeps the fastest pair per stage (ray generation, which only the rasteriser uses,
+ * keeps the default's), then times the wave sizes 2^23, 2^24 and
  * 2^25 (those the budget fills) with the chosen stage shapes and keeps the fastest forward,
  * then two and three chains of waves (branches = 2, 3) at the chosen wave size and at half of
  * it, where the tuned views fill as many waves as chains, kept if faster still. Each shape is
@@ -359,7 +362,9 @@ mirres_status mirres_autotune_wave(mirres_context* ctx, mirres_scene* const* sce
 
 /* Summed device time (ms) and launch count of each stage of the last batched-wavefront
  * render that was issued with params.flags bit 0: out_ms[0..3] = closest hit, shade (RIS),
- * shadow rays, ray generation; out_launches likewise. Synchronises on those events. */
+ * shadow rays, ray generation; out_launches the number of stage spans likewise. Without the rasteriser
+ * (flags bit 2) the ray-generation spans hold no kernel: the closest-hit stage makes the camera rays.
+ * Synchronises on those events. */
 mirres_status mirres_stage_times(mirres_context* ctx, double out_ms[4], int32_t out_launches[4]);
 
 /* The same events one by one, in the order the render issued them: out_ms[i] the device time

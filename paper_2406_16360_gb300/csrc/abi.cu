@@ -1077,7 +1077,7 @@ extern "C" mirres_status mirres_autotune_wave(mirres_context* ctx, mirres_scene*
     int wave_top = 23;
     while (wave_top < 25 && (1ull << wave_top) < sub_total) ++wave_top;
     best.wave_log2 = wave_top;
-    double best_stage[4] = {1e300, 1e300, 1e300, 1e300};
+    double best_stage[3] = {1e300, 1e300, 1e300};
     for (int c = 0; c < n_cand && status == MIRRES_OK; ++c) {
         mirres_wave_shape w = best;
         for (int k = 0; k < 4; ++k) {
@@ -1088,7 +1088,7 @@ extern "C" mirres_status mirres_autotune_wave(mirres_context* ctx, mirres_scene*
         float tot = 0.0f;
         status = run(w, ms, &tot, 1);
         if (status != MIRRES_OK) break;
-        for (int k = 0; k < 4; ++k) {
+        for (int k = 0; k < 3; ++k) {  // (no ray generation without the rasteriser: its span is empty)
             if (ms[k] < best_stage[k]) {
                 best_stage[k] = ms[k];
                 best.block[k] = kCand[c][0];

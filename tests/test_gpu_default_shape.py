@@ -102,3 +102,14 @@ def test_a_tuned_context_is_not_slower_than_an_untuned_one(M):  # noqa: F811
         ratios.append(fastest() / untuned)
     gw.close()
     assert min(ratios) <= 1.02, ratios
+
+
+def test_the_tuner_leaves_ray_generation_alone(M):  # noqa: F811
+    """without the rasteriser no kernel runs in that stage, so there is nothing to choose its shape by"""
+    from paper_2406_16360_gb300.renderer import GpuWorkload
+    gw = GpuWorkload(synth.config2(res=64, n_views=2, tex=16, spp=4), 0)  # below the default's two chains
+    tape = gw.new_tape()
+    for _ in range(4):
+        res = M.mirres_autotune_wave(gw.ctx, [s.handle for s in gw.scenes], gw.views, gw.params(1), tape, 0)
+        assert (res["block"][3], res["blocks_per_sm"][3]) == (256, 8)
+    gw.close()
