@@ -1305,44 +1305,83 @@ __global__ void k_account(unsigned long long* counters, const unsigned int* __re
     atomicAdd(&counters[2], shadow);
 }
 
-// ray queries for mirres_trace through the 8-wide BVH, one ray per thread
-__global__ void __launch_bounds__(256) k_trace_rays_wide(SceneDev s, const float* __restrict__ rays,
-                                                         const int32_t* __restrict__ skip, int64_t n, int any,
+// Whether at least three of four runs of 32 rays, spread over the n, are bundles: neighbouring origins
+// (within a twentieth of the scene's diagonal) and directions within 18 degrees. For blocks of four warps;
+// every block of a launch finds the same.
+__device__ __forceinline__ bool rays_alike(const float* __restrict__ rays, int64_t n, float tmin)
+{
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const float* const r = rays + 6 * (32 * (((n >> 5) - 1) * w / 3) + lane);
+    const float3 o = f3(r[0], r[1], r[2]), d = f3(r[3], r[4], r[5]);
+    const float3 o0 = f3(__shfl_sync(MR_FULL, o.x, 0), __shfl_sync(MR_FULL, o.y, 0), __shfl_sync(MR_FULL, o.z, 0));
+    const float3 d0 = f3(__shfl_sync(MR_FULL, d.x, 0), __shfl_sync(MR_FULL, d.y, 0), __shfl_sync(MR_FULL, d.z, 0));
+    const float c = dot(d, d0), far = 5e3f * tmin;
+    const float3 e = sub(o, o0);
+    const bool near = c > 0.0f && c * c >= 0.9f * dot(d, d) * dot(d0, d0) && dot(e, e) <= far * far;
+    return __syncthreads_count(__all_sync(MR_FULL, near) && lane == 0) >= 3;
+}
+
+template <bool ANY, bool WIDE>
+__device__ __forceinline__ void trace_ray_alone(const SceneDev& s, const float* __restrict__ rays,
+                                                const int32_t* __restrict__ skip, int64_t i,
+                                                int32_t* __restrict__ hit_tri, float* __restrict__ hit_tuv, float tmin,
+                                                uint32_t* sstk)
+{
+    const float3 o = f3(rays[6 * i], rays[6 * i + 1], rays[6 * i + 2]);
+    const float3 d = f3(rays[6 * i + 3], rays[6 * i + 4], rays[6 * i + 5]);
+    Hit h;
+    trace_as<ANY, WIDE>(s, o, d, skip ? skip[i] : -1, tmin, __int_as_float(0x7f800000), h, sstk);
+    hit_tri[i] = ANY ? (h.tri >= 0 ? 1 : -1) : h.tri;
+    if (!ANY && hit_tuv) {
+        hit_tuv[3 * i] = h.tri >= 0 ? h.t : 0.0f;
+        hit_tuv[3 * i + 1] = h.u;
+        hit_tuv[3 * i + 2] = h.v;
+    }
+}
+
+// ray queries for mirres_trace, one ray per thread: through the 8-wide BVH, and where no lane gets a second ray
+template <bool ANY, bool WIDE>
+__global__ void __launch_bounds__(256) k_trace_rays_each(SceneDev s, const float* __restrict__ rays,
+                                                         const int32_t* __restrict__ skip, int64_t n,
                                                          int32_t* __restrict__ hit_tri, float* __restrict__ hit_tuv)
 {
     extern __shared__ __align__(16) uint32_t sstk[];
     const float tmin = *s.tmin_dev;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const float3 o = f3(rays[6 * i], rays[6 * i + 1], rays[6 * i + 2]);
-        const float3 d = f3(rays[6 * i + 3], rays[6 * i + 4], rays[6 * i + 5]);
-        const int sk = skip ? skip[i] : -1;
-        Hit h;
-        if (any) trace_as<true, true>(s, o, d, sk, tmin, __int_as_float(0x7f800000), h, sstk + threadIdx.x);
-        else trace_as<false, true>(s, o, d, sk, tmin, __int_as_float(0x7f800000), h, sstk + threadIdx.x);
-        hit_tri[i] = any ? (h.tri >= 0 ? 1 : -1) : h.tri;
-        if (hit_tuv && !any) {
-            hit_tuv[3 * i] = h.tri >= 0 ? h.t : 0.0f;
-            hit_tuv[3 * i + 1] = h.u;
-            hit_tuv[3 * i + 2] = h.v;
-        }
-    }
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        trace_ray_alone<ANY, WIDE>(s, rays, skip, i, hit_tri, hit_tuv, tmin, sstk + threadIdx.x);
 }
 
-// Ray queries through the binary tree: a caller's rays come in any order, so the lanes of a warp are
-// handed new rays as theirs end and leaves are put aside (trav_warp), as for the renderer's
-// continuation rays. A warp takes every (warps of the grid)-th run of 32 rays, so no counter has to
-// be kept. A million rays (closest, then any) on 50k triangles: 881 us with one ray
-// per thread, now 586.
+// Ray queries through the binary tree, more of them than lanes in flight. In any order: the lanes of a warp
+// are handed new rays as theirs end and leaves are put aside (trav_warp), as for the renderer's continuation
+// rays; a warp of the first `pool_blocks` blocks, one resident wave, takes every (warps of the wave)-th run of
+// 32 rays, so no counter has to be kept. In bundles (a camera's rays in pixel order, its shadow rays): the rays
+// of a warp end together, refilling only mixes distant ones, and putting leaves aside delays the nearer hit;
+// they are traced one per thread by small blocks, handed out as SMs have room.
+// A million rays, closest / any, us, one ray per thread by 256-thread blocks, refilled whatever the order, now:
+// random, 50k triangles 487 / 417, 306 / 289, 300 / 283; camera order, 2k 125 / 110, 179 / 152, 121 / 94; 50k
+// 280 / 257, 300 / 273, 222 / 194; 500k 436 / 406, 390 / 349, 357 / 309. Just above one ray a lane: 200k in
+// camera order, 50k 84 / 81, 111 / 102, 91 / 82; random 149 / 137, 138 / 130, 140 / 134.
+// (Whole rounds of bundles by the resident wave and only the last by further blocks: 600k in camera order 213
+// instead of 160. The blocks behind the wave cost a refilled million 1%: each looks at the rays and ends.)
+constexpr int TR_BLOCK = 128;
 template <bool ANY>
-__global__ void __launch_bounds__(256, 4) k_trace_rays(SceneDev s, const float* __restrict__ rays,
-                                                       const int32_t* __restrict__ skip, int64_t n,
-                                                       int32_t* __restrict__ hit_tri, float* __restrict__ hit_tuv)
+__global__ void __launch_bounds__(TR_BLOCK, 1024 / TR_BLOCK) k_trace_rays(SceneDev s, const float* __restrict__ rays,
+                                                                          const int32_t* __restrict__ skip, int64_t n,
+                                                                          unsigned pool_blocks,
+                                                                          int32_t* __restrict__ hit_tri,
+                                                                          float* __restrict__ hit_tuv)
 {
     extern __shared__ __align__(16) uint32_t sstk[];
-    uint32_t lstk[MR_LSTACK];
     const float tmin = *s.tmin_dev;
+    if (rays_alike(rays, n, tmin)) {
+        for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+            trace_ray_alone<ANY, false>(s, rays, skip, i, hit_tri, hit_tuv, tmin, sstk + threadIdx.x);
+        return;
+    }
+    if (blockIdx.x >= pool_blocks) return;
+    uint32_t lstk[MR_LSTACK];
     const bool ahead = trav_ahead(s);
-    const int64_t step = (int64_t)gridDim.x * blockDim.x;
+    const int64_t step = (int64_t)pool_blocks * blockDim.x;
     int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u), pool = base;  // [pool, end): the run's rest
     int64_t end = min(base + 32, n);
     Trav T;
@@ -1601,13 +1640,16 @@ void mr_launch_l2(const float* img, const float* ref, int64_t n, float* dimg, fl
 void mr_launch_trace_rays(const SceneDev& s, const float* rays, const int32_t* skip, int64_t n, int any,
                           int32_t* hit_tri, float* hit_tuv, int sms, cudaStream_t st)
 {
-    if (s.wnodes) {
-        k_trace_rays_wide<<<grid_cap((uint64_t)n, 256, sms * 8), 256, stack_bytes(256), st>>>(s, rays, skip, n, any,
-                                                                                              hit_tri, hit_tuv);
+    // Up to one ray a lane (1024 threads an SM) there is nothing to refill a lane with, and putting leaves
+    // aside only costs: 1000 random rays, closest, 84 us refilled and 76 one per thread (50k triangles), 155k of
+    // them 121 and 108, 199 and 166 on 500k triangles.
+    if (s.wnodes || n <= (int64_t)sms * 1024) {
+        const auto k = s.wnodes ? (any ? k_trace_rays_each<true, true> : k_trace_rays_each<false, true>)
+                                : (any ? k_trace_rays_each<true, false> : k_trace_rays_each<false, false>);
+        k<<<grid_cap((uint64_t)n, 256, sms * 8), 256, stack_bytes(256), st>>>(s, rays, skip, n, hit_tri, hit_tuv);
         return;
     }
-    const size_t smem = sizeof(uint32_t) * (MR_SSTACK + MR_PEND) * 256;
-    const unsigned grid = grid_cap((uint64_t)n, 256, sms * 4);  // one resident wave
-    if (any) k_trace_rays<true><<<grid, 256, smem, st>>>(s, rays, skip, n, hit_tri, hit_tuv);
-    else k_trace_rays<false><<<grid, 256, smem, st>>>(s, rays, skip, n, hit_tri, hit_tuv);
+    const size_t smem = sizeof(uint32_t) * (MR_SSTACK + MR_PEND) * TR_BLOCK;
+    (any ? k_trace_rays<true> : k_trace_rays<false>)<<<grid_cap((uint64_t)n, TR_BLOCK, sms * 32), TR_BLOCK, smem, st>>>(
+        s, rays, skip, n, sms * (1024 / TR_BLOCK), hit_tri, hit_tuv);
 }
