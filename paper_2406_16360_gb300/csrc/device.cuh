@@ -1190,10 +1190,9 @@ __device__ __forceinline__ unsigned lanemask_lt() { return (1u << lane_id()) - 1
 // each key's lanes in lane order, every key at once: ceil(log2(largest group)) steps of
 // NV + 1 shuffles, however many distinct keys the warp holds.
 template <int NV, class Emit>
-__device__ __forceinline__ void scatter_agg(int key, const float (&v)[NV], const Emit& emit)
+__device__ __forceinline__ void scatter_agg(int key, unsigned peers, const float (&v)[NV], const Emit& emit)
 {
     const int lane = lane_id();
-    const unsigned peers = __match_any_sync(MR_FULL, key);
     const unsigned after = peers & ~((2u << lane) - 1u);  // my key's lanes above me
     int nxt = (key >= 0 && after) ? __ffs(after) - 1 : -1;
     float acc[NV];
@@ -1210,4 +1209,9 @@ __device__ __forceinline__ void scatter_agg(int key, const float (&v)[NV], const
         nxt = nxt >= 0 ? n2 : -1;
     }
     if (key >= 0 && (__ffs(peers) - 1) == lane) emit(key, acc);
+}
+template <int NV, class Emit>
+__device__ __forceinline__ void scatter_agg(int key, const float (&v)[NV], const Emit& emit)
+{
+    scatter_agg<NV>(key, __match_any_sync(MR_FULL, key), v, emit);
 }

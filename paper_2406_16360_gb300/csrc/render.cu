@@ -892,7 +892,7 @@ __global__ void __launch_bounds__(256, MR_BWD_MINB) k_backward(const SceneDev* _
                     const unsigned same = __match_any_sync(MR_FULL, ek);
                     auto emit_env = [&](int t, const float (&x)[3]) { red4(gd.penv + t, x[0], x[1], x[2], 0.0f); };
                     if (__any_sync(MR_FULL, ek >= 0 && __popc(same) > 2)) {
-                        scatter_agg<3>(ek, env_v, emit_env);
+                        scatter_agg<3>(ek, same, env_v, emit_env);
                     } else {
                         const unsigned other = same & ~(1u << lane_id());
                         const int from = other ? __ffs(other) - 1 : lane_id();
