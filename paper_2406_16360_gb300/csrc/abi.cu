@@ -1230,9 +1230,10 @@ static mirres_status backward_impl(mirres_context* ctx, mirres_scene* const* sce
     std::vector<GradDev> gdev((size_t)n_scenes);
     // Packed materials and gradient accumulators cost about 160 bytes of traffic per texel and 60
     // per env texel and vertex, for packing, zeroing and adding up, and three more launches; they
-    // save 15 to 30 ps a sample. One view, us a call, direct / packed: 512 x 512 textures 43 / 54 at
-    // 2^18 samples, 66 / 75 at 2^19, 230 / 215 at 2^21; 1000 x 1000 and 131k env texels 68 / 113 at
-    // 2^19, 239 / 228 at 2^21. The line lies between: 2^20 samples, and one per parameter.
+    // save 10 to 30 ps a sample. One view, us a call, direct / packed: 512 x 512 textures 74 / 77 at
+    // 2^18 samples, 97 / 93 at 2^19, 152 / 135 at 2^20, 272 / 225 at 2^21; 1000 x 1000 and 131k env
+    // texels 98 / 123 at 2^19, 161 / 167 at 2^20, 275 / 249 at 2^21. The line lies there: 2^20 samples,
+    // and one per parameter.
     // Accumulators are kept for the destinations that are asked for only.
     struct AccCounts {
         size_t tex, env, verts;  // records: two float4 a texel, one an env texel or a vertex

@@ -207,21 +207,8 @@ __device__ __forceinline__ float sub_hi(uint32_t x) { return ((float)(x >> 16) +
 __device__ __forceinline__ float sub_lo(uint32_t x) { return ((float)(x & 0xFFFFu) + 0.5f) * 1.52587890625e-5f; }
 
 // ---------------------------------------------------------------------------------------
-// environment map: lookup and inverse-CDF sampling over uint32 thresholds
+// environment map: lookup and inverse-CDF sampling over 53-bit thresholds
 // ---------------------------------------------------------------------------------------
-// largest i in [0, n-1] with a[i] <= k (a[0] == 0 <= k)
-__device__ __forceinline__ int search_le(const uint32_t* __restrict__ a, int n, uint32_t k)
-{
-    int lo = 0, len = n;
-    while (len > 1) {
-        const int half = len >> 1;
-        const int mid = lo + half;
-        if (__ldg(a + mid) <= k) lo = mid;
-        len -= half;
-    }
-    return lo;
-}
-
 __device__ __forceinline__ int env_texel_of(const SceneDev& s, float3 d)
 {
     const float u = atan2f(d.x, -d.z) * (0.5f * MR_INV_PI) + 0.5f;
