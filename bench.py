@@ -555,7 +555,7 @@ def main():
                 "ms_denoise_fwd_bwd": ms_dn, "pixels": pix, "levels": 3, "sigmas": list(EAWT_SIGMAS),
                 "roofline": {"bound": "hbm", "achieved": ach, "peak": HBM_PEAK, "unit": "GB/s",
                              "frac": ach / HBM_PEAK, "traffic": None, "bytes_per_pixel": bytes_px,
-                             "kernel": "k_eawt_level + k_eawt_level_adjoint",
+                             "kernel": "k_eawt_level (forward and adjoint)",
                              "launches_per_level": 1 if uniform else len(gw.views),
                              "peak_basis": "hbm_gbs of MEASURED_PEAKS.json"}}
 
@@ -752,7 +752,7 @@ def main():
                    "shadow": 12.0 * work[2] + 27.0 * work[3]}
     names = {"shade": "k_wshade (shade + RIS stage)",
              "closest": "k_wclosest + k_wclosest_refill (closest-hit stage: primary, then continuation rays)",
-             "shadow": "k_wshadow (shadow-ray stage)"}
+             "shadow": "k_wshadow_refill (shadow-ray stage)"}
     units_per_render = {"closest": (cnt_b[0] + cnt_b[1]) / args.steps, "shade": cand_per_render,
                         "shadow": cnt_b[2] / args.steps}
     traffic_ok = _traffic_valid()
