@@ -81,8 +81,8 @@ __device__ __forceinline__ void store3(float* o3, uint32_t p, float x, float y, 
 // (about 29 instructions a tap and output: nine differences, the squared distances, one
 // exponential, the sums) and its code size: the four rows that both outputs use are a loop, not
 // unrolled, as the flat 6 x 5 x 2 body overran the instruction cache (20% of the stalls).
-// 8 images of 800 x 800, three levels, forward / adjoint: 851 / 1097 us with flat strips of two
-// (unrolled, three 16-byte loads a tap and 1 / k read per tap), now 575 / 705.
+// Calls on 8 images of 800 x 800, three levels, forward / adjoint: 939 / 1125 us with flat strips of two
+// (unrolled, three 16-byte loads a tap and 1 / k read per tap), now 687 / 727.
 // ADJOINT: gout(q) = sum over taps of h w(q, q + tap) gin(q + tap) / k(q + tap), the weights recomputed
 // from the level's recorded input c, 1 / k in gin's fourth word; the output carries the next level's
 // (ikio). Forward: cout = sum h w c / k, and 1 / k to ikio.
